@@ -7,6 +7,7 @@
 #include "sc32.cuh"
 #include "sc32_tma.cuh"
 #include "sc32w.cuh"
+#include "sc64.cuh"
 
 #include <stdlib.h>
 #include <string.h>
@@ -56,13 +57,39 @@ static cudaError_t launch_one(const StepParams& p, int grid, int block,
   return cudaGetLastError();
 }
 
+// FP64-arithmetic kernel: 128-thread blocks (up to 255 registers, two
+// blocks per SM), or one warp per block while that spreads the nodes over
+// more SMs: the FP64 pipes then see one warp each instead of four blocks'
+// worth on a few SMs.
+template <class L, class T, int MODE, int DIAG>
+static cudaError_t launch_sc64(const StepParams& p, cudaStream_t s,
+                               int* grid_used) {
+  auto k = k_sc64<L, T, MODE, DIAG>;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long warps = (p.n + 31) / 32;
+  const int block = warps <= 4LL * sms ? 32 : 128;
+  const int grid = block == 32 ? (int)warps
+                               : occupancy_grid(k, block, p.n);
+  if (grid_used) *grid_used = grid;
+  k<<<grid, block, 0, s>>>(p);
+  count_launch();
+  return cudaGetLastError();
+}
+
 template <class L, class T, int MODE>
 static cudaError_t launch_diag(int diag, int check, const StepParams& p,
                                int grid, int block, cudaStream_t s,
                                int* grid_used) {
   if (check) return launch_one<L, T, MODE, 1, 1>(p, grid, block, s, grid_used);
-  if (diag) return launch_one<L, T, MODE, 1, 0>(p, grid, block, s, grid_used);
-  return launch_one<L, T, MODE, 0, 0>(p, grid, block, s, grid_used);
+  if constexpr (L::D == 1) {
+    if (diag) return launch_one<L, T, MODE, 1, 0>(p, grid, block, s, grid_used);
+    return launch_one<L, T, MODE, 0, 0>(p, grid, block, s, grid_used);
+  } else {
+    if (diag) return launch_sc64<L, T, MODE, 1>(p, s, grid_used);
+    return launch_sc64<L, T, MODE, 0>(p, s, grid_used);
+  }
 }
 
 template <class L, class T>

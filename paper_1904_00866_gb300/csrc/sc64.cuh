@@ -1,0 +1,194 @@
+// Stream-collide kernel in FP64 arithmetic: FP64 storage with every alpha
+// mode, FP32 / FP16 storage with ROOT and SECANT.
+//
+// A thread collides one node per iteration, consecutive threads consecutive
+// nodes of the flat index (ragged rows leave no lane idle).  Nodes near
+// equilibrium take the series path (series64.cuh: ~120 FP64 instructions
+// per D3Q27 FORMULA node and 60 per D2Q9 node, at 64 cycles each the
+// kernel's bound: FP64 pipe 84 % busy for D2Q9), the others re-gather
+// their populations and take the logarithm path (node_fp64.cuh) out of
+// line, so that its registers do not count here.
+//
+// Measured (GB300, us per step; before: every node through the logarithm
+// path, one row segment of 32 nodes per warp, ~700 FP64 instructions per
+// D2Q9 FORMULA node):
+//   D2Q9 1024^2 shear layer, FP64 storage, FORMULA     1326 ->  128
+//   D2Q9 1024^2 shear layer, FP32 storage, ROOT       11560 ->  565
+//   D3Q27 128^3 Taylor-Green, FP64 storage, FORMULA    7960 ->  667
+//   D2Q9 64^2, FP64 storage, FORMULA with statistics     69 ->   12
+// Populations after 8 to 54 steps are as far from the 64-bit reference as
+// before or nearer (1.3e-15 against 1.4e-15 on 128^3).
+#pragma once
+#include "fp16_storage.cuh"
+#include "series64.cuh"
+#include "stats.cuh"
+#include "stream_collide.cuh"
+
+namespace elbm {
+
+// Stored value of population i as FP64, and the inverse.
+template <class L, class T>
+__device__ __forceinline__ double load64(T v, int i, double rho0,
+                                         bool unshifted) {
+  if constexpr (sizeof(T) == 8) {
+    return v;
+  } else if constexpr (sizeof(T) == 2) {
+    return fma(L::w(i), rho0, f2d(__half2float(v) * L::hscale_inv(i)));
+  } else {
+    const double d = f2d(v);
+    return unshifted ? d : fma(L::w(i), rho0, d);
+  }
+}
+
+// What the statistics need of one collided node.
+struct Collided64 {
+  double rho, j[3], alpha;
+  unsigned flags;
+  int iters;
+};
+
+template <class L>
+__device__ __forceinline__ void pull_sources(const StepParams& p,
+                                             unsigned node, int& x, int& y,
+                                             int& z) {
+  const unsigned q1 = p.div_nx.div(node);
+  x = (int)(node - q1 * (unsigned)p.nx);
+  const unsigned q2 = p.div_ny.div(q1);
+  y = (int)(q1 - q2 * (unsigned)p.ny);
+  z = (int)q2;
+}
+
+// The logarithm path of one node, from its stored values in f_in.  Flags
+// NF_BAD_*: the state is invalid and the node is copied unchanged.
+template <class L, class T, int MODE>
+__device__ __noinline__ Collided64 far64_node(const StepParams& p,
+                                              unsigned node) {
+  const T* __restrict__ fin = static_cast<const T*>(p.f_in);
+  T* __restrict__ fout = static_cast<T*>(p.f_out);
+  int x, y, z;
+  pull_sources<L>(p, node, x, y, z);
+  Node64<L> nd;
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const T v = fin[(long long)i * p.ps + src_index<L>(p, i, x, y, z)];
+    if constexpr (sizeof(T) == 8)
+      nd.f[i] = v;
+    else if constexpr (sizeof(T) == 2)
+      nd.f[i] = h16_to_f<L>(v, i, p.rho0);
+    else
+      nd.f[i] = p.unshifted ? (double)v : L::w(i) * p.rho0 + (double)v;
+  }
+  Collided64 r;
+  r.iters = 0;
+  r.alpha = 2.0;
+  r.flags = node64_prepare(nd);
+  r.rho = nd.rho;
+  r.j[0] = nd.j[0];
+  r.j[1] = nd.j[1];
+  r.j[2] = nd.j[2];
+  const bool bad = r.flags != 0;
+  double ab = 0.0;
+  if (!bad) {
+    r.alpha = node64_alpha<L, MODE>(nd, p.secant_iters, r.flags, r.iters);
+    if (sizeof(T) != 8) r.alpha = (double)__double2float_rd(r.alpha);
+    ab = r.alpha * p.beta;
+  } else {
+    atomicOr(p.err_flags, r.flags);
+  }
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const double val =
+        bad ? nd.f[i] : fma(ab, nd.f[i] * nd.x[i], nd.f[i]);
+    T& out = fout[(long long)i * p.ps + node];
+    if constexpr (sizeof(T) == 8)
+      out = val;
+    else if constexpr (sizeof(T) == 2)
+      out = h16_from_dev<L>(val - L::w(i) * p.rho0, i);
+    else
+      out = (T)(p.unshifted ? val : val - L::w(i) * p.rho0);
+  }
+  return r;
+}
+
+template <class L, class T, int MODE, int DIAG>
+__global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
+  constexpr int Q = L::Q;
+  const T* __restrict__ fin = static_cast<const T*>(p.f_in);
+  T* __restrict__ fout = static_cast<T*>(p.f_out);
+  Acc acc;
+  if (DIAG) acc.init();
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < p.n;
+       k += (long long)gridDim.x * blockDim.x) {
+    const unsigned node = (unsigned)k;
+    Near64<L> nd;
+    {
+      int x, y, z;
+      pull_sources<L>(p, node, x, y, z);
+      // element offsets of the neighbours along each axis
+      const int dx[3] = {x == p.nx - 1 ? 1 - p.nx : 1, 0,
+                         x == 0 ? p.nx - 1 : -1};
+      const long long rx = p.nx, pl = (long long)p.nx * p.ny;
+      const long long dy[3] = {y == p.ny - 1 ? rx * (1 - p.ny) : rx, 0,
+                               y == 0 ? rx * (p.ny - 1) : -rx};
+      const long long dz[3] = {z == p.nz - 1 ? pl * (1 - p.nz) : pl, 0,
+                               z == 0 ? pl * (p.nz - 1) : -pl};
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const long long src = k + dx[L::c(i, 0) + 1] + dy[L::c(i, 1) + 1] +
+                              (L::D == 3 ? dz[L::c(i, 2) + 1] : 0);
+        nd.f[i] = load64<L, T>(fin[(long long)i * p.ps + src], i, p.rho0,
+                               p.unshifted);
+      }
+    }
+    Series64 se;
+    if (near64_prepare(nd, se)) {
+      unsigned flags = 0;
+      int iters = 0;
+      double alpha = 2.0;
+      if (se.rest)
+        flags = NF_DEGENERATE;
+      else if (MODE == MODE_ROOT)
+        alpha = alpha_root_near(nd, se, flags, iters);
+      else if (MODE == MODE_SECANT)
+        alpha = alpha_secant_near(se, p.secant_iters, flags, iters);
+      else
+        alpha = alpha_formula_near(se, flags);
+      if (sizeof(T) != 8) alpha = (double)__double2float_rd(alpha);
+      const double ab = alpha * p.beta;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const double val = fma(ab, nd.n[i], nd.f[i]);
+        T& out = fout[(long long)i * p.ps + k];
+        if constexpr (sizeof(T) == 8)
+          out = val;
+        else if constexpr (sizeof(T) == 2)
+          out = h16_from_dev<L>(fma(-L::w(i), p.rho0, val), i);
+        else
+          out = (T)(p.unshifted ? val : fma(-L::w(i), p.rho0, val));
+      }
+      if (p.alpha_map) p.alpha_map[k] = (float)alpha;
+      if (DIAG) {
+        const double j[3] = {nd.j[0] * nd.unit, nd.j[1] * nd.unit,
+                             L::D == 3 ? nd.j[2] * nd.unit : 0.0};
+        // 1/2 rho |u|^2 with u = j / rho in the node's units
+        const double ke = nd.unit * nd.inv_rho *
+                          (nd.j[0] * nd.j[0] + nd.j[1] * nd.j[1] +
+                           nd.j[2] * nd.j[2]);
+        acc.add_moments_ke(fma(nd.rho, nd.unit, -p.rho0), j, 0.5 * ke);
+        acc.add_alpha(alpha, flags, iters);
+      }
+    } else {
+      const Collided64 c = far64_node<L, T, MODE>(p, node);
+      if (!(c.flags & (NF_BAD_NEG | NF_BAD_NONFINITE))) {
+        if (p.alpha_map) p.alpha_map[k] = (float)c.alpha;
+        if (DIAG) {
+          acc.add_moments(c.rho - p.rho0, c.j, c.rho);
+          acc.add_alpha(c.alpha, c.flags, c.iters);
+        }
+      }
+    }
+  }
+  if (DIAG) acc.block_reduce_store(p.partials);
+}
+
+}  // namespace elbm
