@@ -146,11 +146,11 @@ typedef struct {
   long long n_accept_star;  /* alpha_* accepted (any alpha_*)             */
   long long n_formula;      /* Eq. (9) / secant / root alpha used         */
   long long n_band;         /* FP32 FORMULA: FP32 decision not certified,
-                               decided by the double-float second stage   */
+                               decided by the double-float second stage
+                               or, what that leaves open, the FP64 series */
   long long n_far;          /* FP32 FORMULA: node solved in FP64 (far from
-                               equilibrium, invalid, or undecided by the
-                               second stage and its double-float series
-                               pass)                                      */
+                               equilibrium, invalid, or Delta H(2) within
+                               its rounding of zero)                      */
   long long n_degenerate;   /* f^eq == f: alpha = 2                       */
   long long n_root_iters;   /* ROOT/SECANT iterations                     */
   long long n_root_cap;     /* ROOT stopped at the iteration cap          */

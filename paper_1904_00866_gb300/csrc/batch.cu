@@ -188,7 +188,7 @@ struct elbm_batch {
   size_t tmem_cap = 0;
   int* d_count = nullptr;
   MemberStats* d_stats = nullptr;
-  unsigned* d_far_count = nullptr;   // [2] deferred nodes by step parity
+  unsigned* d_far_count = nullptr;   // [4] deferred and open nodes
   float* d_refine = nullptr;         // undecided-node buffer
   unsigned refine_cap = 0;
   unsigned* d_refine_counts = nullptr;   // entries per batch-kernel block
@@ -398,7 +398,7 @@ static elbm_status upload_tables(elbm_batch* b) {
     e = cudaMemcpyAsync(b->d_count, &count, sizeof(int),
                         cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(b->d_far_count, 0, 2 * sizeof(unsigned), b->stream);
+    e = cudaMemsetAsync(b->d_far_count, 0, 4 * sizeof(unsigned), b->stream);
   // the sources are pageable host memory: each copy is staged before the
   // call returns, so the host tables may be rebuilt right away
   if (e != cudaSuccess) return bfail(b, ELBM_ECUDA, cudaGetErrorString(e));
@@ -427,7 +427,7 @@ static cudaError_t run_steps(elbm_batch* b, int nsteps, int diag, int grid) {
   // autotuner's dry steps, which all run as step 0, would never clear
   // counter 0 and its stale entries would pile up.
   cudaError_t e0 =
-      cudaMemsetAsync(b->d_far_count, 0, 2 * sizeof(unsigned), b->stream);
+      cudaMemsetAsync(b->d_far_count, 0, 4 * sizeof(unsigned), b->stream);
   if (e0 != cudaSuccess) return e0;
   for (int s = 0; s < nsteps; ++s) {
     bp.step = s;

@@ -59,7 +59,7 @@ struct BatchParams {
   MemberStats* stats;           // [kBatchMaxMembers]
   unsigned long long* far_queue;   // (member << 32) | node
   unsigned far_cap;
-  unsigned* far_count;          // [2]
+  unsigned* far_count;          // [4], as StepParams::far_count
   unsigned* err_flags;
   int step;                     // step index within the burst
   // undecided nodes for the second stage: records of kBatchRecord floats
@@ -325,8 +325,7 @@ __device__ __forceinline__ void member_stats_add(const BatchParams& bp, int mi,
 
 // Second stage of the undecided nodes the batch kernel (`blocks` blocks)
 // buffered, two blocks per SM; a node it leaves undecided joins the
-// deferred-node queue for the fixup that follows (tagged when the
-// double-float series pass may still decide it).
+// open-node list (the queue's upper end) for the fixup that follows.
 template <int DIAG>
 __global__ void __launch_bounds__(256, 2) k_batch_refine(const BatchParams bp,
                                                          int blocks) {
@@ -375,17 +374,16 @@ __global__ void __launch_bounds__(256, 2) k_batch_refine(const BatchParams bp,
       }
       float (&vq)[L::Q] = *reinterpret_cast<float (*)[L::Q]>(v);
       auto out32 = [&](int i, float val) { out[(size_t)i * m.n + node] = val; };
-      return refine_deferred<L, true, DIAG, 0, false>(pp, vq, node, ap, acc,
-                                                      out32);
+      return refine_deferred<L, true, DIAG, 0>(pp, vq, node, ap, acc, out32);
     };
     const int st = m.lattice == 1 ? run(D3Q27{}) : run(D2Q9{});
     if (st != kStageDone) {
-      // kStageRetry: tagged, so that the fixup (whose register budget
-      // holds it) runs the double-float series pass before any FP64
-      const unsigned q = atomicAdd(&bp.far_count[bp.step & 1], 1u);
+      const int open = st == kStageRetry;
+      const unsigned q =
+          atomicAdd(&bp.far_count[2 * open + (bp.step & 1)], 1u);
       if (q < bp.far_cap)
-        bp.far_queue[q] = ((unsigned long long)mi << 32) |
-                          (node | (st == kStageRetry ? kTagRefine : 0u));
+        bp.far_queue[open ? bp.far_cap - 1u - q : q] =
+            ((unsigned long long)mi << 32) | node;
       else
         atomicOr(bp.err_flags, NF_BAD_NONFINITE);   // cannot happen
     } else if (DIAG) {
@@ -394,15 +392,17 @@ __global__ void __launch_bounds__(256, 2) k_batch_refine(const BatchParams bp,
   }
 }
 
-// FP64 fixup of the batch kernel's deferred-node queue (values gathered
-// from the member's buffer): the second stage for entries tagged
-// kTagRefine (a full buffer segment), one entry per thread, then the FP64
-// FORMULA for the nodes that need it, one node per warp
-// (formula64_warp); entries are dealt as in k_far_fixup.  Clears the other
-// parity's counter for the next step.
+// FP64 fixup of the batch kernel's deferred nodes (values gathered from the
+// member's buffer): both lists as in k_far_fixup.  Clears the other parity's
+// counters for the next step.
 template <int DIAG>
 __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
   const unsigned count = min(bp.far_count[bp.step & 1], bp.far_cap);
+  const unsigned open_count =
+      min(bp.far_count[2 + (bp.step & 1)], bp.far_cap);
+  if (blockIdx.x == 0 && threadIdx.x < 2)
+    bp.far_count[2 * threadIdx.x + ((bp.step & 1) ^ 1)] = 0u;
+  if (count + open_count == 0u) return;
   const int lane = threadIdx.x & 31;
   const unsigned W = gridDim.x * (blockDim.x >> 5);
   const unsigned wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -410,9 +410,11 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
   const bool bulk = count > gridDim.x * blockDim.x;
   auto coords = [](const MemberDesc& m, unsigned node, int& x, int& y,
                    int& z) {
-    x = (int)(node % (unsigned)m.nx);
-    y = (int)((node / (unsigned)m.nx) % (unsigned)m.ny);
-    z = (int)(node / ((unsigned)m.nx * (unsigned)m.ny));
+    const unsigned q1 = m.div_nx.div(node);
+    x = (int)(node - q1 * (unsigned)m.nx);
+    const unsigned q2 = m.div_ny.div(q1);
+    y = (int)(q1 - q2 * (unsigned)m.ny);
+    z = (int)q2;
   };
   auto params = [&](const MemberDesc& m) {
     StepParams pp;
@@ -464,8 +466,8 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
       run(D2Q9{});
     if (DIAG) member_stats_add(bp, mi, m, acc, true);
   };
-  // FP64 FORMULA of queue entry ee by the whole warp (every lane calls)
-  auto fp64_warp = [&](unsigned long long ee) {
+  // FP64 FORMULA of queue entry ee by the whole warp, as in k_far_fixup
+  auto fp64_warp = [&](unsigned long long ee, bool near) {
     const int mi = (int)(ee >> 32);
     const unsigned node = (unsigned)(ee & 0xffffffffu) & ~kTagRefine;
     const MemberDesc& m = bp.members[mi];
@@ -473,6 +475,7 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
     float* out = pick(m, m.parity0 + bp.step + 1);
     int x, y, z;
     coords(m, node, x, y, z);
+    bool settled = false;
     auto run = [&](auto lat, const LanePop& lp) {
       using L = decltype(lat);
       double f = 0.0;
@@ -486,9 +489,13 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
             (size_t)xs;
         f = lp.w * m.rho0 + (double)in[(size_t)lane * m.n + src];
       }
-      return formula64_warp<L>(lp, f, m.beta64, [&](double val) {
+      auto store = [&](double val) {
         out[(size_t)lane * m.n + node] = (float)(val - lp.w * m.rho0);
-      });
+      };
+      Warp64 w;
+      settled = near && near64_warp<L>(lp, lane, f, m.beta64, w, store);
+      if (!settled) w = formula64_warp<L>(lp, f, m.beta64, store);
+      return w;
     };
     const Warp64 r = m.lattice == 1 ? run(D3Q27{}, lp27) : run(D2Q9{}, lp9);
     if (lane == 0) {
@@ -501,94 +508,173 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
           acc.init();
           acc.add_moments(r.rho - m.rho0, r.j, r.rho);
           acc.add_alpha(r.alpha, r.flags, 0);
-          member_stats_add(bp, mi, m, acc, true);
+          member_stats_add(bp, mi, m, acc, !settled);
         }
       }
     }
   };
-  __shared__ unsigned long long pend_s[8][32];   // 256 threads: 8 warps
-  unsigned long long* pend = pend_s[threadIdx.x >> 5];
-  int npend = 0;
+  // FP64 series FORMULA of entry ee in this thread; false: not settled
+  auto near_lane = [&](unsigned long long ee) {
+    const int mi = (int)(ee >> 32);
+    const unsigned node = (unsigned)(ee & 0xffffffffu) & ~kTagRefine;
+    const MemberDesc& m = bp.members[mi];
+    const float* in = pick(m, m.parity0 + bp.step);
+    float* out = pick(m, m.parity0 + bp.step + 1);
+    StepParams g;   // geometry for src_index
+    g.nx = m.nx;
+    g.ny = m.ny;
+    g.nz = m.nz;
+    int x, y, z;
+    coords(m, node, x, y, z);
+    auto run = [&](auto lat) {
+      using L = decltype(lat);
+      Near64<L> nd;
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i)
+        nd.f[i] = load64<L, float>(
+            in[(size_t)i * m.n + src_index<L>(g, i, x, y, z)], i, m.rho0,
+            false);
+      double alpha = 2.0;
+      unsigned flags = NF_BAND;
+      if (!near64_formula(nd, alpha, flags)) return false;
+      const double ab = alpha * m.beta64;
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i) {
+        const double val = fma(ab, nd.n[i], nd.f[i]);
+        out[(size_t)i * m.n + node] = (float)fma(-L::w(i), m.rho0, val);
+      }
+      if (m.alpha_map) m.alpha_map[node] = (float)alpha;
+      if (DIAG) {
+        Acc acc;
+        acc.init();
+        const double j[3] = {nd.j[0] * nd.unit, nd.j[1] * nd.unit,
+                             nd.j[2] * nd.unit};
+        const double rho = nd.rho * nd.unit;
+        acc.add_moments(rho - m.rho0, j, rho);
+        acc.add_alpha(alpha, flags, 0);
+        member_stats_add(bp, mi, m, acc, false);
+      }
+      return true;
+    };
+    return m.lattice == 1 ? run(D3Q27{}) : run(D2Q9{});
+  };
+  __shared__ unsigned long long pend_s[8][32], near_s[8][64];
+  const int warp = threadIdx.x >> 5;
+  unsigned long long* pend = pend_s[warp];
+  unsigned long long* near = near_s[warp];
+  int npend = 0, nnear = 0;
   auto flush = [&]() {   // every lane calls
     __syncwarp();
     if (lane < npend) fp64_lane(pend[lane]);
     __syncwarp();
     npend = 0;
   };
-  for (unsigned base = 0; base < count; base += 32u * W) {
-    const unsigned k = base + (unsigned)lane * W + wid;
-    bool need64 = false;
-    unsigned long long e = 0;
-    if (k < count) {
-      e = bp.far_queue[k];
-      const int mi = (int)(e >> 32);
-      const unsigned tagged = (unsigned)(e & 0xffffffffu);
-      const unsigned node = tagged & ~kTagRefine;
-      need64 = true;
-      if (tagged & kTagRefine) {
-        const MemberDesc& m = bp.members[mi];
-        const float* in = pick(m, m.parity0 + bp.step);
-        float* out = pick(m, m.parity0 + bp.step + 1);
-        StepParams g;   // geometry for src_index
-        g.nx = m.nx;
-        g.ny = m.ny;
-        g.nz = m.nz;
-        int x, y, z;
-        coords(m, node, x, y, z);
-        Acc acc;
-        acc.init();
-        const StepParams pp = params(m);
-        auto run = [&](auto lat) {
-          using L = decltype(lat);
-          float v[L::Q];
-#pragma unroll
-          for (int i = 0; i < L::Q; ++i)
-            v[i] = in[(size_t)i * m.n + src_index<L>(g, i, x, y, z)];
-          auto store32 = [&](int i, float val) {
-            out[(size_t)i * m.n + node] = val;
-          };
-          const float nan = __int_as_float(0x7fc00000);
-          int st = refine_deferred<L, true, DIAG, 0, false>(pp, v, node, nan,
-                                                            acc, store32);
-          // as in k_far_fixup: no series pass on a queue longer than the grid
-          if (st == kStageRetry && !bulk)
-            st = refine_deferred<L, true, DIAG, 0, true>(pp, v, node, nan,
-                                                         acc, store32);
-          return st == kStageDone;
-        };
-        need64 = !(m.lattice == 1 ? run(D3Q27{}) : run(D2Q9{}));
-        if (DIAG && !need64) member_stats_add(bp, mi, m, acc, false);
-      }
-    }
-    // FP64 nodes of this round, as in k_far_fixup: one per warp for a few,
-    // one per lane for many; a queue longer than the grid (new members'
-    // first steps) collects them per warp and runs them 32 at a time
-    const unsigned todo = __ballot_sync(0xffffffffu, need64);
-    if (!bulk && __popc(todo) > 16) {
+  auto logarithms = [&](bool need64, unsigned long long e, bool near) {
+    const unsigned m64 = __ballot_sync(0xffffffffu, need64);
+    if (!bulk && !near && __popc(m64) > 16) {
       if (need64) fp64_lane(e);
-    } else if (bulk) {
-      const int nk = __popc(todo);
+    } else if (bulk && !near) {
+      const int nk = __popc(m64);
       if (npend + nk > 32) flush();
-      if (need64) pend[npend + __popc(todo & ((1u << lane) - 1u))] = e;
+      if (need64) pend[npend + __popc(m64 & ((1u << lane) - 1u))] = e;
       npend += nk;
     } else {
-      unsigned m = todo;
+      unsigned m = m64;
       while (m) {
         const int src_lane = __ffs(m) - 1;
         m &= m - 1;
-        fp64_warp(__shfl_sync(0xffffffffu, e, src_lane));
+        fp64_warp(__shfl_sync(0xffffffffu, e, src_lane), near);
       }
     }
+  };
+  // rounds as in k_far_fixup
+  const unsigned use = open_warps(open_count, gridDim.x);
+  const unsigned WO = gridDim.x * use;
+  const unsigned run_o = run_length(open_count, WO);
+  const unsigned run_q = run_length(count, W);
+  unsigned base_o = (unsigned)warp < use ? 0u : open_count, base_q = 0u;
+  for (;;) {
+    bool need64 = false, open = false, direct = false;
+    unsigned long long e = 0;
+    if (base_o < open_count) {
+      const unsigned k = base_o +
+                         (blockIdx.x * use + (unsigned)warp) * run_o +
+                         (unsigned)lane;
+      base_o += run_o * WO;
+      direct = (unsigned)lane < run_o && k < open_count;
+      if (direct) e = bp.far_queue[bp.far_cap - 1u - k];
+    } else if (base_q < count) {
+      const unsigned k = base_q + wid * run_q + (unsigned)lane;
+      base_q += run_q * W;
+      if ((unsigned)lane < run_q && k < count) {
+        e = bp.far_queue[k];
+        const int mi = (int)(e >> 32);
+        const unsigned tagged = (unsigned)(e & 0xffffffffu);
+        const unsigned node = tagged & ~kTagRefine;
+        need64 = true;
+        if (tagged & kTagRefine) {
+          const MemberDesc& m = bp.members[mi];
+          const float* in = pick(m, m.parity0 + bp.step);
+          float* out = pick(m, m.parity0 + bp.step + 1);
+          StepParams g;   // geometry for src_index
+          g.nx = m.nx;
+          g.ny = m.ny;
+          g.nz = m.nz;
+          int x, y, z;
+          coords(m, node, x, y, z);
+          Acc acc;
+          acc.init();
+          const StepParams pp = params(m);
+          auto run = [&](auto lat) {
+            using L = decltype(lat);
+            float v[L::Q];
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i)
+              v[i] = in[(size_t)i * m.n + src_index<L>(g, i, x, y, z)];
+            auto store32 = [&](int i, float val) {
+              out[(size_t)i * m.n + node] = val;
+            };
+            const float nan = __int_as_float(0x7fc00000);
+            return refine_deferred<L, true, DIAG, 0>(pp, v, node, nan, acc,
+                                                     store32);
+          };
+          const int st = m.lattice == 1 ? run(D3Q27{}) : run(D2Q9{});
+          open = st == kStageRetry;
+          need64 = st == kStageFP64;
+          if (DIAG && st == kStageDone)
+            member_stats_add(bp, mi, m, acc, false);
+        }
+      }
+    } else if (nnear == 0) {
+      break;
+    }
+    const unsigned mo = __ballot_sync(0xffffffffu, open);
+    if (open) near[nnear + __popc(mo & ((1u << lane) - 1u))] = e;
+    nnear += __popc(mo);
+    unsigned long long sn = e;
+    if (nnear >= 32 || (nnear > 0 && base_q >= count)) {
+      const int take = min(nnear, 32);
+      nnear -= take;
+      __syncwarp();
+      direct = lane < take;
+      if (direct) sn = near[nnear + lane];
+      __syncwarp();
+    }
+    const bool few =
+        __popc(__ballot_sync(0xffffffffu, direct)) <= kFewOpen;
+    if (!few) direct = direct && !near_lane(sn);
+#pragma unroll 1
+    for (int t = 0; t < 2; ++t)
+      logarithms(t == 0 ? direct : need64, t == 0 ? sn : e, t == 0 && few);
   }
   if (npend > 0) {   // bulk remainder: few nodes run one per warp
     __syncwarp();
     if (npend > 5) {
       flush();
     } else {
-      for (int j = 0; j < npend; ++j) fp64_warp(pend[j]);
+      for (int j = 0; j < npend; ++j) fp64_warp(pend[j], false);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) bp.far_count[(bp.step & 1) ^ 1] = 0u;
 }
 
 }  // namespace elbm

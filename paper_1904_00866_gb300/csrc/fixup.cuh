@@ -6,15 +6,16 @@
 //     recomputed in double-float arithmetic, the decision retaken with its
 //     much smaller error bound (node32_refine), and the populations the
 //     decided alpha changes rewritten.
-//   k_far_fixup: the FP64 FORMULA (Eqs. (8)-(9) with logarithms, alpha
-//     rounded down to FP32; one node per warp) for nodes far from
-//     equilibrium (max |x_i| > 1/8, a velocity component >= 1/4), invalid
-//     states and the rare node the second stage left undecided.  It also
-//     resets the other parity's counter for the next step (stream order
-//     makes that counter idle here).
+//   k_far_fixup: two lists of deferred nodes.  What the second stage left
+//     open takes the FP64 series FORMULA (near64_formula), one node per
+//     lane.  Nodes far from equilibrium (max |x_i| > 1/8, a velocity
+//     component >= 1/4), invalid states and the rare node the series does
+//     not settle take the FP64 FORMULA with logarithms, one node per warp.
+//     alpha is rounded down to FP32.  It also resets the other parity's
+//     counters for the next step (stream order makes them idle here).
 #pragma once
-#include <type_traits>
 #include "sc32.cuh"
+#include "series64.cuh"
 #include "warp64.cuh"
 
 namespace elbm {
@@ -22,15 +23,15 @@ namespace elbm {
 // Second stage of one deferred node from its stored values v[] (FP32
 // storage: the stored value; FP16: the decoded deviation); the kernel wrote
 // it with the provisional alpha ap (NaN: unknown, recomputed).  Returns
-// the second stage's status (kStageDone, kStageRetry: run again with DFS,
-// kStageFP64: left to the FP64 path).
-template <class L, bool SHIFTED, int DIAG, int CHECK, bool DFS, class Out>
+// the second stage's status (kStageDone, kStageRetry: left to the FP64
+// series, kStageFP64: left to the logarithms).
+template <class L, bool SHIFTED, int DIAG, int CHECK, class Out>
 __device__ __forceinline__ int refine_deferred(const StepParams& p,
                                                const float (&v)[L::Q],
                                                long long node, float ap,
                                                Acc& acc, Out out) {
   auto in = [&](int i) { return v[i]; };
-  return second_stage32<L, SHIFTED, DIAG, CHECK, DFS>(
+  return second_stage32<L, SHIFTED, DIAG, CHECK>(
       in, p.rho0f, p.betaf, p.corr_rho, p.corr,
       p.alpha_map ? p.alpha_map + node : nullptr, ap, out,
       [&](const N32<L>& r) {
@@ -54,10 +55,8 @@ __device__ __forceinline__ int refine_deferred(const StepParams& p,
 // every block of this kernel forms their prefix sums in shared memory and
 // takes entries k with a grid stride.  The double-float stage decides (and
 // rewrites the populations its alpha changes); the few nodes its FP32
-// series leaves open join the deferred-node queue tagged, so that the
-// fixup (whose register budget holds it) runs them again with the leading
-// terms of the series in double-float and collides the rest in FP64 with
-// a whole warp.
+// series leaves open join the open-node list (the queue's upper end), for
+// the FP64 series in the fixup, whose register budget holds it.
 template <class L, class S, int DIAG, int CHECK>
 __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
                                                          int blocks) {
@@ -98,7 +97,7 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
     const float ap = w[Q + 1];
     int st;
     if constexpr (sizeof(S) == 2) {
-      st = refine_deferred<L, true, DIAG, CHECK, false>(
+      st = refine_deferred<L, true, DIAG, CHECK>(
           p, v, node, ap, acc, [&](int i, float val) {
             reinterpret_cast<unsigned short*>(p.out_pop[i])[node] =
                 h16_bits<L>(val, i);
@@ -106,18 +105,17 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
     } else {
       auto out = [&](int i, float val) { p.out_pop[i][node] = val; };
       st = shifted
-               ? refine_deferred<L, true, DIAG, CHECK, false>(p, v, node, ap,
+               ? refine_deferred<L, true, DIAG, CHECK>(p, v, node, ap,
                                                               acc, out)
-               : refine_deferred<L, false, DIAG, CHECK, false>(p, v, node, ap,
+               : refine_deferred<L, false, DIAG, CHECK>(p, v, node, ap,
                                                                acc, out);
     }
     if (st != kStageDone) {
-      // kStageRetry: tagged, so that the fixup runs the double-float
-      // series pass (in its larger register budget) before any FP64
-      const unsigned q = atomicAdd(&p.far_count[p.parity], 1u);
+      // still open: list from the queue's top; far: list from its bottom
+      const int open = st == kStageRetry;
+      const unsigned q = atomicAdd(&p.far_count[2 * open + p.parity], 1u);
       if (q < p.far_cap)
-        p.far_queue[q] =
-            (unsigned)node | (st == kStageRetry ? kTagRefine : 0u);
+        p.far_queue[open ? p.far_cap - 1u - q : q] = (unsigned)node;
       else
         atomicOr(p.err_flags, NF_BAD_NONFINITE);   // cannot happen: cap = n
     }
@@ -125,22 +123,79 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
   if (DIAG) acc.block_reduce_store(p.partials);
 }
 
-// FP64 fixup (S: the storage type, float or half_t): the deferred-node
-// queue, with values gathered from f_in.  Entries tagged kTagRefine (a
-// full buffer segment, or no buffer) take the second stage here first, one
-// entry per thread; the nodes that need the FP64 FORMULA are then collided
-// one at a time by their whole warp (formula64_warp, one population per
-// lane).  Lane l of warp w takes entry w + l W of each round of 32 W
-// entries (W warps in the grid), so a short queue leaves at most a few
-// FP64 nodes to each warp and a long one (the first step after
-// initialisation) still gives every lane its own entry; a warp with more
-// than 16 FP64 nodes in a round runs them one per lane.  On steps with the
-// FP64 entropy check (CHECK) the FP64 nodes run on their own lanes, as the
-// check's statistics need each node's populations in one thread.
+// FP64 fixup (S: the storage type, float or half_t); values are gathered
+// from f_in.  The open-node list (what the second stage left) takes the FP64
+// series, one node per lane.  Of the deferred-node queue, entries tagged
+// kTagRefine (a full buffer segment, or no buffer) take the second stage
+// here first, one per thread, and what it leaves is collected per warp for
+// the series.  Nodes that need the logarithms are collided one at a time
+// by their whole warp (formula64_warp, one population per lane), or one per
+// lane when a warp has more than 16, collected 32 at a time on a queue
+// longer than the grid (the first step after initialisation).  On steps with
+// the FP64 entropy check (CHECK) they run on their own lanes, as the check's
+// statistics need each node's populations in one thread.
+//
+// Bound by latency: a short list is one chain per warp, and by the fetch of
+// straight-line code that each warp runs once.  A few open nodes run one
+// at a time (near64_warp), many one per lane (near64_formula: up to 32 nodes
+// for ~120 FP64 instructions of 64 cycles).  Before, the second stage ran
+// again with double-float leading terms (~3,000 FP32 instructions) and what
+// that left took the logarithms, ~460 FP64 instructions a node.  Entries are
+// dealt evenly as runs of neighbours; the grid is one block per SM (the
+// kernel's registers allow no second one).
+// us per launch, before -> now (GB300): D3Q27 256^3 binary16 41 -> 15,
+// 121 x 64 x 70 static step (no buffer) 36 -> 22, D2Q9 1024^2 shear layer
+// 25 -> 12; all open nodes one per lane: static 64.
+template <class L>
+__device__ __forceinline__ void near64_gather(const StepParams& p, int x, int y,
+                                              int z, const float*, double (&f)[L::Q]) {
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i)
+    f[i] = load64<L, float>(p.in_pop[i][src_index<L>(p, i, x, y, z)], i,
+                            p.rho0, p.unshifted);
+}
+template <class L>
+__device__ __forceinline__ void near64_gather(const StepParams& p, int x, int y,
+                                              int z, const half_t*, double (&f)[L::Q]) {
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i)
+    f[i] = load64<L, half_t>(reinterpret_cast<const half_t*>(
+                                 p.in_pop[i])[src_index<L>(p, i, x, y, z)],
+                             i, p.rho0, false);
+}
+
+// Entries of a list of `count` that a warp of `warps` takes per round: runs
+// of neighbouring entries, of equal length, at most 32.
+__device__ __forceinline__ unsigned run_length(unsigned count, unsigned warps) {
+  return min(32u, (count + warps - 1u) / warps);
+}
+
+// Open nodes a warp settles one at a time (near64_warp, ~2.5 us each) rather
+// than one per lane (~25 us for D3Q27, ~10 us for D2Q9, however few).
+constexpr int kFewOpen = 8;
+// Warps per block that take open nodes: all while each gets few, then one
+// per sub-partition as long as their lanes hold the list (two would share
+// the FP64 pipe for nothing), then all.
+__device__ __forceinline__ unsigned open_warps(unsigned count,
+                                               unsigned blocks) {
+  return count > blocks * (8u * kFewOpen) && count <= blocks * (4u * 32u) ? 4u
+                                                                          : 8u;
+}
+
 template <class L, class S, int DIAG, int CHECK>
 __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
   constexpr int Q = L::Q;
   const unsigned count = min(p.far_count[p.parity], p.far_cap);
+  const unsigned open_count = min(p.far_count[2 + p.parity], p.far_cap);
+  if (blockIdx.x == 0 && threadIdx.x < 2)
+    p.far_count[2 * threadIdx.x + (p.parity ^ 1)] = 0u;
+  if (count + open_count == 0u) {   // uniform: this row of statistics is empty
+    if (DIAG && threadIdx.x < NSTAT)
+      p.partials[(long long)blockIdx.x * NSTAT + threadIdx.x] =
+          threadIdx.x == S_AMIN ? INFINITY
+                                : (threadIdx.x == S_AMAX ? -INFINITY : 0.0);
+    return;
+  }
   const bool shifted = sizeof(S) == 2 || !p.unshifted;
   const int lane = threadIdx.x & 31;
   const unsigned W = gridDim.x * (blockDim.x >> 5);
@@ -150,9 +205,7 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
   Acc acc;
   acc.init();
   auto coords = [&](long long node, int& x, int& y, int& z) {
-    x = (int)(node % p.nx);
-    y = (int)((node / p.nx) % p.ny);
-    z = (int)(node / ((long long)p.nx * p.ny));
+    node_xyz<L>(p, (unsigned)node, x, y, z);
   };
   auto out_s = [&](long long node, int i, float val) {
     if constexpr (sizeof(S) == 2)
@@ -192,8 +245,9 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
     if (DIAG) acc.far += 1;
     collide64<L, MODE_FORMULA, CHECK>(nd, p, true, acc, DIAG != 0, store_s);
   };
-  // FP64 FORMULA of node nd by the whole warp (every lane calls)
-  auto fp64_warp = [&](long long nd) {
+  // FP64 FORMULA of node nd by the whole warp (every lane calls): the series
+  // form when `near` and it settles the node, else the logarithm form
+  auto fp64_warp = [&](long long nd, bool near) {
     int x, y, z;
     coords(nd, x, y, z);
     double f = 0.0;
@@ -212,15 +266,19 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
       }
       if (shifted) f += lp.w * p.rho0;
     }
-    const Warp64 r = formula64_warp<L>(lp, f, p.beta, [&](double val) {
+    auto store = [&](double val) {
       if constexpr (sizeof(S) == 2)
         reinterpret_cast<half_t*>(p.out_pop[lane])[nd] =
             __double2half((val - lp.w * p.rho0) * (double)lp.hscale);
       else
         p.out_pop[lane][nd] = (float)(p.unshifted ? val : val - lp.w * p.rho0);
-    });
+    };
+    Warp64 r;
+    const bool settled =
+        near && near64_warp<L>(lp, lane, f, p.beta, r, store);
+    if (!settled) r = formula64_warp<L>(lp, f, p.beta, store);
     if (lane == 0) {
-      if (DIAG) acc.far += 1;
+      if (DIAG) acc.far += !settled;
       if (r.flags & (NF_BAD_NEG | NF_BAD_NONFINITE)) {
         atomicOr(p.err_flags, r.flags);
       } else {
@@ -232,68 +290,69 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
       }
     }
   };
-  // bulk queues: this warp's pending FP64 nodes (warp-uniform count)
-  __shared__ unsigned pend_s[8][32];   // 256 threads: 8 warps
-  unsigned* pend = pend_s[threadIdx.x >> 5];
-  int npend = 0;
+  // FP64 series FORMULA of one node in this thread; false: not settled
+  auto near_lane = [&](long long node) {
+    int x, y, z;
+    coords(node, x, y, z);
+    Near64<L> nd;
+    near64_gather<L>(p, x, y, z, static_cast<const S*>(nullptr), nd.f);
+    double alpha = 2.0;
+    unsigned flags = NF_BAND;
+    if (!near64_formula(nd, alpha, flags)) return false;
+    const double ab = alpha * p.beta;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const double val = fma(ab, nd.n[i], nd.f[i]);
+      if constexpr (sizeof(S) == 2)
+        reinterpret_cast<half_t*>(p.out_pop[i])[node] =
+            h16_from_dev<L>(fma(-L::w(i), p.rho0, val), i);
+      else
+        p.out_pop[i][node] =
+            (float)(p.unshifted ? val : fma(-L::w(i), p.rho0, val));
+    }
+    if (p.alpha_map) p.alpha_map[node] = (float)alpha;
+    if (DIAG) {
+      const double j[3] = {nd.j[0] * nd.unit, nd.j[1] * nd.unit,
+                           nd.j[2] * nd.unit};
+      const double rho = nd.rho * nd.unit;
+      acc.add_moments(rho - p.rho0, j, rho);
+      acc.add_alpha(alpha, flags, 0);
+      if (CHECK) {
+        Node64<L> c;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) c.f[i] = nd.f[i];
+        node64_prepare(c);
+        const Check64 ck = node64_check(c, alpha);
+        acc.add_check(ck.h, ck.violation,
+                      decision_mismatch(flags, ck.accept_ref),
+                      fabs(alpha - ck.alpha_ref));
+      }
+    }
+    return true;
+  };
+  // this warp's pending nodes (warp-uniform counts): for the logarithms (on
+  // a queue longer than the grid) and for the series
+  // (8 warps; the series' list is below 32 before a round adds up to 32)
+  __shared__ unsigned pend_s[8][32], near_s[8][64];
+  const int warp = threadIdx.x >> 5;
+  unsigned* pend = pend_s[warp];
+  unsigned* near = near_s[warp];
+  int npend = 0, nnear = 0;
   auto flush = [&]() {   // every lane calls
     __syncwarp();
     if (lane < npend) fp64_lane((long long)pend[lane]);
     __syncwarp();
     npend = 0;
   };
-  for (unsigned base = 0; base < count; base += 32u * W) {
-    const unsigned k = base + (unsigned)lane * W + wid;
-    bool need64 = false;
-    long long node = 0;
-    if (k < count) {
-      const unsigned e = p.far_queue[k];
-      node = e & ~kTagRefine;
-      need64 = true;
-      if (e & kTagRefine) {
-        int x, y, z;
-        coords(node, x, y, z);
-        float v[Q];
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-          const long long src = src_index<L>(p, i, x, y, z);
-          if constexpr (sizeof(S) == 2)
-            v[i] = h16_dev<L>(reinterpret_cast<const unsigned short*>(
-                                  p.in_pop[i])[src],
-                              i);
-          else
-            v[i] = p.in_pop[i][src];
-        }
-        const float ap = __int_as_float(0x7fc00000);   // NaN: recomputed
-        auto out = [&](int i, float val) { out_s(node, i, val); };
-        auto run = [&](auto dfs) {
-          constexpr bool DFS = decltype(dfs)::value;
-          return shifted ? refine_deferred<L, true, DIAG, CHECK, DFS>(
-                               p, v, node, ap, acc, out)
-                         : refine_deferred<L, false, DIAG, CHECK, DFS>(
-                               p, v, node, ap, acc, out);
-        };
-        int st = run(std::false_type{});
-        // the series pass pays off on the few nodes of a developed flow; on
-        // a queue longer than the grid (the first step after
-        // initialisation, where n is rounding noise and the pass decides
-        // few nodes) they go to the FP64 path directly
-        if (st == kStageRetry && !bulk) st = run(std::true_type{});
-        need64 = st != kStageDone;
-      }
-    }
-    // FP64 nodes of this round.  Per lane a node costs ~75 FP64 warp
-    // instructions of its warp (2,400 shared by 32 lanes), per warp ~460:
-    // one per warp ends sooner when a warp has few such nodes (developed
-    // flows), one per lane costs less FP64 issue in bulk.  On a queue
-    // longer than the grid (the first step after initialisation, ~1 % of
-    // the nodes in FP64) each warp collects its FP64 nodes in shared memory
-    // and runs them 32 at a time, one per lane.  The check's statistics
-    // need each node in one thread.
+  // Nodes that need the logarithms (every lane calls).  Per lane a node
+  // costs ~75 FP64 warp instructions of its warp (2,400 shared by 32 lanes),
+  // per warp ~460: one per warp ends sooner when a warp has few such nodes,
+  // one per lane costs less FP64 issue in bulk.
+  auto logarithms = [&](bool need64, long long node, bool near) {
     const unsigned m64 = __ballot_sync(0xffffffffu, need64);
-    if (CHECK != 0 || (!bulk && __popc(m64) > 16)) {
+    if (CHECK != 0 || (!bulk && !near && __popc(m64) > 16)) {
       if (need64) fp64_lane(node);
-    } else if (bulk) {
+    } else if (bulk && !near) {
       const int nk = __popc(m64);
       if (npend + nk > 32) flush();
       if (need64) pend[npend + __popc(m64 & ((1u << lane) - 1u))] =
@@ -304,19 +363,94 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
       while (m) {
         const int src_lane = __ffs(m) - 1;
         m &= m - 1;
-        fp64_warp(__shfl_sync(0xffffffffu, node, src_lane));
+        fp64_warp(__shfl_sync(0xffffffffu, node, src_lane), near);
       }
     }
+  };
+  // Rounds over the open-node list, then over the queue, then until the
+  // nodes its second stage left are settled; one call site each for the
+  // series and the logarithms.
+  const unsigned use = open_warps(open_count, gridDim.x);
+  const unsigned WO = gridDim.x * use;
+  const unsigned run_o = run_length(open_count, WO);
+  const unsigned run_q = run_length(count, W);
+  unsigned base_o = (unsigned)warp < use ? 0u : open_count, base_q = 0u;
+  for (;;) {
+    bool need64 = false, open = false, direct = false;
+    long long node = 0;
+    if (base_o < open_count) {
+      const unsigned k = base_o +
+                         (blockIdx.x * use + (unsigned)warp) * run_o +
+                         (unsigned)lane;
+      base_o += run_o * WO;
+      direct = (unsigned)lane < run_o && k < open_count;
+      if (direct) node = p.far_queue[p.far_cap - 1u - k];
+    } else if (base_q < count) {
+      const unsigned k = base_q + wid * run_q + (unsigned)lane;
+      base_q += run_q * W;
+      if ((unsigned)lane < run_q && k < count) {
+        const unsigned e = p.far_queue[k];
+        node = e & ~kTagRefine;
+        need64 = true;
+        if (e & kTagRefine) {
+          int x, y, z;
+          coords(node, x, y, z);
+          float v[Q];
+#pragma unroll
+          for (int i = 0; i < Q; ++i) {
+            const long long src = src_index<L>(p, i, x, y, z);
+            if constexpr (sizeof(S) == 2)
+              v[i] = h16_dev<L>(reinterpret_cast<const unsigned short*>(
+                                    p.in_pop[i])[src],
+                                i);
+            else
+              v[i] = p.in_pop[i][src];
+          }
+          const float ap = __int_as_float(0x7fc00000);   // NaN: recomputed
+          auto out = [&](int i, float val) { out_s(node, i, val); };
+          const int st =
+              shifted ? refine_deferred<L, true, DIAG, CHECK>(p, v, node, ap,
+                                                              acc, out)
+                      : refine_deferred<L, false, DIAG, CHECK>(p, v, node, ap,
+                                                               acc, out);
+          open = st == kStageRetry;
+          need64 = st == kStageFP64;
+        }
+      }
+    } else if (nnear == 0) {
+      break;
+    }
+    // nodes for the series: this round's list entries, or a warp's worth
+    // (at the end, the rest) of what the second stage left
+    const unsigned mo = __ballot_sync(0xffffffffu, open);
+    if (open)
+      near[nnear + __popc(mo & ((1u << lane) - 1u))] = (unsigned)node;
+    nnear += __popc(mo);
+    long long sn = node;
+    if (nnear >= 32 || (nnear > 0 && base_q >= count)) {   // warp-uniform
+      const int take = min(nnear, 32);
+      nnear -= take;
+      __syncwarp();
+      direct = lane < take;
+      if (direct) sn = (long long)near[nnear + lane];
+      __syncwarp();
+    }
+    // a warp with few such nodes runs them in turn, one population per lane
+    const bool few =
+        CHECK == 0 && __popc(__ballot_sync(0xffffffffu, direct)) <= kFewOpen;
+    if (!few) direct = direct && !near_lane(sn);
+#pragma unroll 1
+    for (int t = 0; t < 2; ++t)
+      logarithms(t == 0 ? direct : need64, t == 0 ? sn : node, t == 0 && few);
   }
   if (npend > 0) {   // bulk remainder: few nodes run one per warp
     __syncwarp();
     if (npend > 5) {
       flush();
     } else {
-      for (int j = 0; j < npend; ++j) fp64_warp((long long)pend[j]);
+      for (int j = 0; j < npend; ++j) fp64_warp((long long)pend[j], false);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) p.far_count[p.parity ^ 1] = 0u;
   if (DIAG) acc.block_reduce_store(p.partials);
 }
 

@@ -329,23 +329,17 @@ __device__ __forceinline__ void exact_moments(float d0,
 // known to 6.1 u |x_i| + G (1 + Dd)^3 2^-37 instead of the FP32 path's
 // equilibrium rounding, and the decision is retaken with the bounds of that
 // accuracy (series always to k = 8).  A node this leaves undecided is
-// flagged NF_FAR | NF_REFINE; the DFS variant then evaluates the leading
-// terms of Delta H(2) in double-float too (its resolution is set by the
-// double-float n, ~1e-12 of W_i rho, instead of the FP32 series' ~75 u),
-// and a node still undecided (NF_FAR) goes to the FP64 fixup.  Writes
+// flagged NF_FAR | NF_REFINE: its Delta H(2) lies within ~75 u of its own
+// scale, and the FP64 series (series64.cuh) settles it.  Writes
 // r.n0 / r.n2 (the more accurate n, used by the relaxation), r.alpha,
 // r.flags (NF_BAND set: the second stage decided) and the moments r.drho,
 // r.rho, r.j.
-template <class L, bool SHIFTED, bool DFS = false>
+template <class L, bool SHIFTED>
 __device__ __forceinline__ void node32_refine(
     float d0, const float2 (&dd)[npairs<L>()], float rho0, float corr_rho,
     const float* __restrict__ corr, float a_extra, N32<L>& r) {
   constexpr int P = npairs<L>();
   constexpr float uu = 5.9604645e-8f;  // 2^-24
-  // DFS: the leading terms -M3/3 + 2 M4/3 of Delta H(2) in double-float as
-  // well (x_i = n_i / f_i as a double-float quotient), for the nodes the
-  // FP32 series on the double-float n leaves undecided
-  DF<float> m3d = {0.0f, 0.0f}, m4d = {0.0f, 0.0f};
   // exact_moments needs sum |delta_i| < 4
   {
     float2 sa = make_float2(fabsf(dd[0].x), fabsf(dd[0].y));
@@ -439,13 +433,6 @@ __device__ __forceinline__ void node32_refine(
       M[k] = pw;
       pw *= x;
     }
-    if (DFS) {
-      const DF<float> fd = df_add(df_mul(wdf(0), rho0), d0);   // f_0
-      const DF<float> xd = df_div(t, fd);
-      const DF<float> n2 = df_mul(df_mul(t, xd), xd);          // f x^3
-      m3d = n2;
-      m4d = df_mul(n2, xd);                                    // f x^4
-    }
   }
   auto pair = [&](int a, int c) { return df_pair(psi[a][c + 1], psi[a][1 - c]); };
   DF<float2> pxy[3][3];
@@ -476,19 +463,6 @@ __device__ __forceinline__ void node32_refine(
     for (int e = 2; e <= 8; ++e) {
       mk[e] = add2(mk[e], pw);
       pw = mul2(pw, x);
-    }
-    if (DFS) {
-      const DF<float2> fd =
-          df_add(df_mul(df_bcast(wdf(i)), f2(rho0)), dd[k]);   // f_i
-      const DF<float2> xd = df_div(t, fd);
-      const DF<float2> n2 = df_mul(df_mul(t, xd), xd);
-      const DF<float2> n3 = df_mul(n2, xd);
-      const DF<float> a3 = df_add(DF<float>{n2.hi.x, n2.lo.x},
-                                  DF<float>{n2.hi.y, n2.lo.y});
-      const DF<float> a4 = df_add(DF<float>{n3.hi.x, n3.lo.x},
-                                  DF<float>{n3.hi.y, n3.lo.y});
-      m3d = df_add(m3d, a3);
-      m4d = df_add(m4d, a4);
     }
   }
 #pragma unroll
@@ -527,40 +501,11 @@ __device__ __forceinline__ void node32_refine(
   const float En = 2.0f * e2u *
                    (G * (opdD * fmaf(3.0f, cpsi, 52.0f) + 33.0f * r0r) + 8.0f);
   const float Ex = 1.01f * (6.1f * uu * xabs + En + G * a_extra);
-  DH32 h = series_dh32<L::Q>(M, true, xabs, Ex, rho.hi);
-  if (DFS) {
-    // Delta H(2) = [-M3 / 3 + 2 M4 / 3] (double-float) + sum_{k=5..8} c_k M_k
-    // (FP32) + tail.  Errors: x_i within Exd = En + G a_extra + 2^-42 |x_i|
-    // (the double-float n, f_i and quotient), propagated through the
-    // leading terms as M2 (1 + 3 xabs) Exd; their double-float rounding
-    // (2,000 u^2 xabs M2 covers 27 terms of a few operations each); the
-    // FP32 terms k = 5..8 from x within Ex (100 u xabs^3 M2 with their
-    // rounding); the tail beyond k = 8; the final FP32 sum.
-    constexpr float c3h = df_hi(-1.0 / 3.0), c3l = df_lo(-1.0 / 3.0);
-    constexpr float c4h = df_hi(2.0 / 3.0), c4l = df_lo(2.0 / 3.0);
-    const DF<float> lead = df_add(df_mul(m3d, DF<float>{c3h, c3l}),
-                                  df_mul(m4d, DF<float>{c4h, c4l}));
-    const float tail =
-        fmaf(-1.1f, M[5],
-             fmaf(26.0f / 15.0f, M[6], fmaf(-19.0f / 7.0f, M[7],
-                                           (30.0f / 7.0f) * M[8])));
-    const float D2 = lead.hi + (lead.lo + tail);
-    const float Exd = 1.01f * (En + G * a_extra + 2.3e-13f * xabs);
-    const float r2 = 2.0f * xabs;
-    const float r2_7 = r2 * r2 * r2 * r2 * r2 * r2 * r2;
-    const float tr2 = __fdividef(r2_7, 18.0f * (1.0f - r2)) * kUp;
-    const float x3 = xabs * xabs * xabs;
-    h.D2 = D2;
-    h.e2 = 1.1f * (M[2] * ((1.0f + 3.0f * xabs) * Exd + 2.0e3f * e2u * xabs +
-                           100.0f * uu * x3 + tr2) +
-                   2.0f * uu * (fabsf(lead.hi) + fabsf(tail)) +
-                   2.0f * rho.hi * (xabs + Exd) * Exd * Exd);
-  }
+  const DH32 h = series_dh32<L::Q>(M, true, xabs, Ex, rho.hi);
   float alpha = 1.0f;
   const int k = decide32(h, alpha, kChordWidth);
   if (k == kUndecided) {
-    // the double-float leading terms (DFS) may still decide it
-    r.flags = DFS ? NF_FAR : (NF_FAR | NF_REFINE);
+    r.flags = NF_FAR | NF_REFINE;
     return;
   }
   r.alpha = alpha;

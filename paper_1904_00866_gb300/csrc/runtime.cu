@@ -131,7 +131,7 @@ struct elbm_handle {
   double* stats_dev = nullptr;
   double* fields = nullptr;   // (1 + D) x n doubles: rho, u staging
   unsigned* err_flags = nullptr;
-  unsigned* far_count = nullptr;   // [0..1] deferred, [2..3] undecided
+  unsigned* far_count = nullptr;   // [0..1] deferred, [2..3] open
   unsigned* far_queue = nullptr;
   float* refine_buf = nullptr;     // undecided-node records [cap][rec]
   unsigned refine_cap = 0;
@@ -607,7 +607,7 @@ elbm_status elbm_step(elbm_handle* h, long long nsteps, elbm_alpha_mode mode) {
   p.refine_counts = h->refine_counts;
   // the deferred-node counters start every call at zero; within the call
   // each step's fixup clears the counter the next step uses
-  if (nsteps > 0) cudaMemsetAsync(h->far_count, 0, 2 * sizeof(unsigned),
+  if (nsteps > 0) cudaMemsetAsync(h->far_count, 0, 4 * sizeof(unsigned),
                                   h->stream);
   const bool d2 = h->lattice == ELBM_D2Q9;
   // 0: FP64, 1: FP32 (shifted or not), 2: FP16-shifted
@@ -671,10 +671,11 @@ elbm_status elbm_step(elbm_handle* h, long long nsteps, elbm_alpha_mode mode) {
     int rows = grid;
     if (fp32_formula) {
       StepParams pf = p;
-      // the second stage and the fixup run at most 2 blocks per SM
-      // (their register budgets), so a larger grid only adds waves of
-      // blocks with nothing to do
+      // the second stage runs 2 blocks per SM and the fixup one (their
+      // register budgets), so a larger grid only adds waves of blocks with
+      // nothing to do
       const int fgrid = std::min(grid, max_grid_rows() / 4);
+      const int xgrid = std::min(grid, max_grid_rows() / 8);
       if (p.exact && p.refine_cap) {
         // second stage of the undecided nodes the step buffered
         pf.partials = h->partials + (size_t)rows * NSTAT;
@@ -692,13 +693,13 @@ elbm_status elbm_step(elbm_handle* h, long long nsteps, elbm_alpha_mode mode) {
       }
       pf.partials = h->partials + (size_t)rows * NSTAT;
       if (storage == 2)
-        e = d2 ? launch_far16_d2q9(diag, check, pf, fgrid, h->stream)
-               : launch_far16_d3q27(diag, check, pf, fgrid, h->stream);
+        e = d2 ? launch_far16_d2q9(diag, check, pf, xgrid, h->stream)
+               : launch_far16_d3q27(diag, check, pf, xgrid, h->stream);
       else
-        e = d2 ? launch_far_d2q9(diag, check, pf, fgrid, h->stream)
-               : launch_far_d3q27(diag, check, pf, fgrid, h->stream);
+        e = d2 ? launch_far_d2q9(diag, check, pf, xgrid, h->stream)
+               : launch_far_d3q27(diag, check, pf, xgrid, h->stream);
       if (e != cudaSuccess) return cuda_fail(h, e, "far fixup launch");
-      rows += fgrid;
+      rows += xgrid;
     }
     if (diag) {
       launch_finish(h->partials, rows, h->stats_dev, h->stream);

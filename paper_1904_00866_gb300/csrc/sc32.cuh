@@ -306,12 +306,12 @@ __device__ __forceinline__ unsigned sc32_node_in(
 // population the decided alpha does not change at storage precision keeps
 // the provisional value, which differs from it by at most the rounding of
 // the FP32 n.  Returns kStageDone, kStageRetry (still undecided by the FP32
-// series on the double-float n: the DFS pass, which also evaluates the
-// leading terms in double-float, may decide it) or kStageFP64 (left to the
-// FP64 path, which rewrites all of it).  Nothing is written unless done.
+// series on the double-float n: the FP64 series rewrites all of it) or
+// kStageFP64 (left to the logarithm form, which does too).  Nothing is
+// written unless done.
 enum { kStageDone = 0, kStageRetry = 1, kStageFP64 = 2 };
-template <class L, bool SHIFTED, int DIAG, int CHECK, bool DFS, class In,
-          class Out, class Stat>
+template <class L, bool SHIFTED, int DIAG, int CHECK, class In, class Out,
+          class Stat>
 __device__ __forceinline__ int second_stage32(In in, float rho0f, float beta,
                                               float corr_rho,
                                               const float* __restrict__ corr,
@@ -330,7 +330,7 @@ __device__ __forceinline__ int second_stage32(In in, float rho0f, float beta,
   N32<L> t;
   t.flags = 0u;
   t.alpha = 1.0f;
-  node32_refine<L, SHIFTED, DFS>(d0, dd, rho0f, corr_rho, corr, a_extra, t);
+  node32_refine<L, SHIFTED>(d0, dd, rho0f, corr_rho, corr, a_extra, t);
   if (t.flags & NF_FAR)
     return (t.flags & NF_REFINE) ? kStageRetry : kStageFP64;
   if (t.alpha != ap)

@@ -26,20 +26,6 @@
 
 namespace elbm {
 
-// Stored value of population i as FP64, and the inverse.
-template <class L, class T>
-__device__ __forceinline__ double load64(T v, int i, double rho0,
-                                         bool unshifted) {
-  if constexpr (sizeof(T) == 8) {
-    return v;
-  } else if constexpr (sizeof(T) == 2) {
-    return fma(L::w(i), rho0, f2d(__half2float(v) * L::hscale_inv(i)));
-  } else {
-    const double d = f2d(v);
-    return unshifted ? d : fma(L::w(i), rho0, d);
-  }
-}
-
 // What the statistics need of one collided node.
 struct Collided64 {
   double rho, j[3], alpha;

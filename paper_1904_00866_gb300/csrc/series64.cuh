@@ -32,6 +32,7 @@
 // the largest, invalid states) report false and take the logarithm path.
 #pragma once
 #include "df32.cuh"
+#include "fp16_storage.cuh"
 #include "node_fp32.cuh"
 #include "node_fp64.cuh"
 
@@ -75,6 +76,20 @@ __device__ __forceinline__ DF<float> split_df(double v, int adj) {
       __uint_as_float(base | ((l & 0x1fffffffu) >> 6)) - __uint_as_float(base);
   const bool in = a >= (25 << 20);
   return {in ? __uint_as_float(hb) : 0.0f, in ? lo : 0.0f};
+}
+
+// Stored value of population i as FP64.
+template <class L, class T>
+__device__ __forceinline__ double load64(T v, int i, double rho0,
+                                         bool unshifted) {
+  if constexpr (sizeof(T) == 8) {
+    return v;
+  } else if constexpr (sizeof(T) == 2) {
+    return fma(L::w(i), rho0, f2d(__half2float(v) * L::hscale_inv(i)));
+  } else {
+    const double d = f2d(v);
+    return unshifted ? d : fma(L::w(i), rho0, d);
+  }
 }
 
 __host__ __device__ constexpr double pow6(int d) {
@@ -365,6 +380,27 @@ __device__ __forceinline__ double alpha_formula_near(const Series64& r,
   if (!(den.hi > 0.0f)) return 1.0;   // f == f^eq to rounding
   const DF<float> t = df_div(D2, den);
   return (2.0 - f2d(t.hi)) - f2d(t.lo);
+}
+
+// The FORMULA of a node the FP32 stages left open (FP32 / FP16 storage): the
+// series decision, taken only where the logarithm form (node_fp64.cuh,
+// warp64.cuh) takes the same branch, and alpha rounded down to FP32.  The
+// logarithm form's Delta H(2) is off by less than 100 u M_2 = 1.1e-14 M_2
+// (u = 2^-53; 27 terms f phi(2 x) of at most 2 f x^2, the products f x L,
+// and x off by 20 u), the series' by less than 20 u M_2, so a value beyond
+// 2^-45 M_2 has the same sign in both, and the two alphas differ by less
+// than 1e-13.  False: out of the series' range, at rest, or within that
+// distance of zero -- the logarithm form decides.
+template <class L>
+__device__ __forceinline__ bool near64_formula(Near64<L>& s, double& alpha,
+                                               unsigned& flags) {
+  Series64 r;
+  if (!near64_prepare(s, r) || r.rest) return false;
+  const float d = __int_as_float((127 + r.e_d) << 23);
+  const DF<float> b2 = series_sum<3, true>(r, d);
+  if (!(fabsf(b2.hi) * d > 2.842170943040401e-14f * r.m[2].hi)) return false;
+  alpha = (double)__double2float_rd(alpha_formula_near(r, flags));
+  return true;
 }
 
 // Delta H(alpha) = alpha (sum_k A_k alpha^(k-1) - T) for alpha <= 4, with

@@ -25,7 +25,7 @@ namespace {
 
 constexpr unsigned kStaticMaxNodes = 1u << 21;   // 2,097,152 lattice nodes
 constexpr int kStaticMaxRows = 4096;             // diagnostic partial rows
-constexpr size_t kCountersBytes = 256;           // far_count[2], err_flags
+constexpr size_t kCountersBytes = 256;           // far_count[4], err_flags
 constexpr size_t kPartialsBytes = sizeof(double) * NSTAT * kStaticMaxRows;
 constexpr size_t kStatsBytes = 256;              // NSTAT doubles, padded
 constexpr size_t kQueueBytes = sizeof(unsigned) * kStaticMaxNodes;
@@ -125,7 +125,7 @@ extern "C" elbm_status elbm_step_static(
   }
   p.alpha_map = alpha_out_device;
   p.partials = partials;
-  p.err_flags = counters + 2;
+  p.err_flags = counters + 4;
   p.far_count = counters;
   p.far_queue = queue;
   p.far_cap = (unsigned)n;
@@ -171,7 +171,7 @@ extern "C" elbm_status elbm_step_static(
   e = cudaMemcpyAsync(slots, stats, sizeof(slots), cudaMemcpyDeviceToHost,
                       stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&flags, counters + 2, sizeof(unsigned),
+    e = cudaMemcpyAsync(&flags, counters + 4, sizeof(unsigned),
                         cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return fail(ELBM_ECUDA, cudaGetErrorString(e));

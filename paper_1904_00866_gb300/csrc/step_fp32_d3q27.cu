@@ -1,4 +1,4 @@
-// D3Q27: FP32-storage certified FORMULA kernels and the FP64 far-node fixup.
+// D3Q27: FP32-storage certified FORMULA kernels.
 #include "launch_step.cuh"
 
 namespace elbm {
@@ -7,13 +7,5 @@ cudaError_t launch_fp32_formula_d3q27(int diag, int check, const StepParams& p,
                                       int* grid_used) {
   (void)block;
   return launch_sc32<D3Q27>(diag, check, p, grid, s, grid_used);
-}
-cudaError_t launch_far_d3q27(int diag, int check, const StepParams& p, int grid,
-                             cudaStream_t s) {
-  return launch_far_lattice<D3Q27>(diag, check, p, grid, s);
-}
-cudaError_t launch_refine_d3q27(int diag, int check, const StepParams& p,
-                                int blocks, int grid, cudaStream_t s) {
-  return launch_refine_lattice<D3Q27>(diag, check, p, blocks, grid, s);
 }
 }  // namespace elbm

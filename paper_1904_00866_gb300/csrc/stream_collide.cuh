@@ -81,7 +81,9 @@ struct StepParams {
   float corr_rho;         // unshifted: sum_i fl(W_i rho0) - rho0
   float corr[27];         // unshifted: W_i rho0 - fl(W_i rho0)
   int secant_iters;
-  unsigned* far_count;    // [2] deferred-node counters, indexed by parity
+  unsigned* far_count;    // [4] by step parity: [0..1] deferred nodes (from
+                          // the queue's bottom), [2..3] nodes the second
+                          // stage left open (from its top)
   unsigned* far_queue;    // node indices deferred to the FP64 fixup
   unsigned far_cap;       // capacity of far_queue (entries)
   int parity;             // step parity selecting far_count[parity]
