@@ -14,6 +14,7 @@
 //     alpha is rounded down to FP32.  It also resets the other parity's
 //     counters for the next step (stream order makes them idle here).
 #pragma once
+#include <type_traits>
 #include "sc32.cuh"
 #include "series64.cuh"
 #include "warp64.cuh"
@@ -25,26 +26,30 @@ namespace elbm {
 // it with the provisional alpha ap (NaN: unknown, recomputed).  Returns
 // the second stage's status (kStageDone, kStageRetry: left to the FP64
 // series, kStageFP64: left to the logarithms).
-template <class L, bool SHIFTED, int DIAG, int CHECK, class Out>
+template <class L, bool SHIFTED, int DIAG, int CHECK, class A, class Out>
 __device__ __forceinline__ int refine_deferred(const StepParams& p,
                                                const float (&v)[L::Q],
-                                               long long node, float ap,
-                                               Acc& acc, Out out) {
+                                               long long node, float ap, A& acc,
+                                               Out out) {
   auto in = [&](int i) { return v[i]; };
   return second_stage32<L, SHIFTED, DIAG, CHECK>(
       in, p.rho0f, p.betaf, p.corr_rho, p.corr,
       p.alpha_map ? p.alpha_map + node : nullptr, ap, out,
       [&](const N32<L>& r) {
         if (!DIAG) return;
-        const double j[3] = {r.j[0], r.j[1], r.j[2]};
-        acc.add_moments((double)r.drho, j, (double)r.rho);
-        acc.add_alpha((double)r.alpha, r.flags, 0);
-        if (CHECK) {
-          Node64<L> nd;
-          const Check64 ck = check32<L, SHIFTED>(in, p.rho0, r.alpha, nd);
-          acc.add_check(ck.h, ck.violation,
-                        decision_mismatch(r.flags, ck.accept_ref),
-                        fabs((double)r.alpha - ck.alpha_ref));
+        if constexpr (std::is_same<A, Acc32>::value) {
+          diag32<L, SHIFTED, CHECK>(r, in, p.rho0, acc);
+        } else {
+          const double j[3] = {r.j[0], r.j[1], r.j[2]};
+          acc.add_moments((double)r.drho, j, (double)r.rho);
+          acc.add_alpha((double)r.alpha, r.flags, 0);
+          if (CHECK) {
+            Node64<L> nd;
+            const Check64 ck = check32<L, SHIFTED>(in, p.rho0, r.alpha, nd);
+            acc.add_check(ck.h, ck.violation,
+                          decision_mismatch(r.flags, ck.accept_ref),
+                          fabs((double)r.alpha - ck.alpha_ref));
+          }
         }
       });
 }
@@ -66,7 +71,10 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
   const unsigned total = pre[blocks];
   const unsigned seg = p.refine_cap / (unsigned)blocks;
   const bool shifted = sizeof(S) == 2 || !p.unshifted;
-  Acc acc;
+  // compensated FP32 sums, as in the stream-collide kernels: FP64 ones (with
+  // their division) take ~25 instructions of 64 cycles per node (32^3 with
+  // statistics on every step: 41 -> 36 us per step)
+  Acc32 acc;
   acc.init();
   for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < total;
        k += gridDim.x * blockDim.x) {
@@ -120,7 +128,7 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
         atomicOr(p.err_flags, NF_BAD_NONFINITE);   // cannot happen: cap = n
     }
   }
-  if (DIAG) acc.block_reduce_store(p.partials);
+  if (DIAG) store_acc32(acc, p.partials);
 }
 
 // FP64 fixup (S: the storage type, float or half_t); values are gathered

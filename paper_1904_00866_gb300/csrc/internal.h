@@ -44,11 +44,6 @@ void stats_from_slots(const double* slots, double rho0, long long n,
                                         cudaStream_t s, int* grid_used);      \
   cudaError_t launch_far16_##LAT(int diag, int check, const StepParams& p,   \
                                  int grid, cudaStream_t s);                  \
-  cudaError_t launch_refine_##LAT(int diag, int check, const StepParams& p,  \
-                                  int blocks, int grid, cudaStream_t s);     \
-  cudaError_t launch_refine16_##LAT(int diag, int check,                     \
-                                    const StepParams& p, int blocks,         \
-                                    int grid, cudaStream_t s);               \
   cudaError_t launch_fp16_fp64mode_##LAT(int mode, int diag, int check,      \
                                          const StepParams& p, int grid,       \
                                          int block, cudaStream_t s,           \
@@ -56,6 +51,13 @@ void stats_from_slots(const double* slots, double rho0, long long n,
 ELBM_DECLARE_LAUNCHERS(d2q9)
 ELBM_DECLARE_LAUNCHERS(d3q27)
 #undef ELBM_DECLARE_LAUNCHERS
+
+// Second stage of the undecided D3Q27 nodes a step buffered (D2Q9 kernels
+// run it themselves).
+cudaError_t launch_refine_d3q27(int diag, int check, const StepParams& p,
+                                int blocks, int grid, cudaStream_t s);
+cudaError_t launch_refine16_d3q27(int diag, int check, const StepParams& p,
+                                  int blocks, int grid, cudaStream_t s);
 
 cudaError_t launch_fp64_d1q3(int mode, int diag, int check,
                              const StepParams& p, int grid, int block,

@@ -228,28 +228,24 @@ static elbm_status ensure_buffers(elbm_handle* h) {
   h->far_count = (unsigned*)dev_alloc(h, 256);
   if (h->dtype != ELBM_FP64) {
     h->far_queue = (unsigned*)dev_alloc(h, sizeof(unsigned) * h->n);
-    // Undecided nodes of a step: about 1-3 % of a developed 3D flow, but
-    // most nodes of a flow whose non-equilibrium part is near FP32
-    // resolution (a thin shear layer at Re 30,000) and of the first step
-    // after initialisation; a full buffer sends the rest to the gathering
-    // queue, where each node costs ~3x more (gather, FP32 stage again).
-    // D2Q9: every node (48-byte records); D3Q27: half the nodes, at most
-    // 2^26 records (8.6 GB) unless n / 16 is more, at least 65,536.
-    const long long cap =
-        h->q == 9
-            ? h->n
-            : std::min<long long>(
-                  h->n, std::max<long long>(
-                            65536, std::min<long long>(
-                                       h->n / 2,
-                                       std::max<long long>(h->n / 16,
-                                                           1LL << 26))));
-    const int rec = h->q == 27 ? refine_record<D3Q27>() : refine_record<D2Q9>();
-    h->refine_buf =
-        (float*)dev_alloc(h, sizeof(float) * (size_t)rec * (size_t)cap);
-    h->refine_counts =
-        (unsigned*)dev_alloc(h, sizeof(unsigned) * kMaxRefineBlocks);
-    h->refine_cap = h->refine_buf && h->refine_counts ? (unsigned)cap : 0u;
+    // Undecided nodes of a D3Q27 step: about 1-3 % of a developed flow, but
+    // most nodes of the first step after initialisation; a full buffer
+    // sends the rest to the gathering queue, where each node costs ~3x more
+    // (gather, FP32 stage again).  Half the nodes, at most 2^26 records
+    // (8.6 GB) unless n / 16 is more, at least 65,536.  D2Q9 kernels run
+    // the second stage themselves.
+    if (h->q == 27) {
+      const long long cap = std::min<long long>(
+          h->n, std::max<long long>(
+                    65536, std::min<long long>(
+                               h->n / 2, std::max<long long>(h->n / 16,
+                                                             1LL << 26))));
+      h->refine_buf = (float*)dev_alloc(
+          h, sizeof(float) * (size_t)refine_record<D3Q27>() * (size_t)cap);
+      h->refine_counts =
+          (unsigned*)dev_alloc(h, sizeof(unsigned) * kMaxRefineBlocks);
+      h->refine_cap = h->refine_buf && h->refine_counts ? (unsigned)cap : 0u;
+    }
   }
   if (!h->f[0] || !h->f[1] || !h->partials || !h->stats_dev ||
       !h->err_flags || !h->far_count ||
@@ -679,15 +675,10 @@ elbm_status elbm_step(elbm_handle* h, long long nsteps, elbm_alpha_mode mode) {
       if (p.exact && p.refine_cap) {
         // second stage of the undecided nodes the step buffered
         pf.partials = h->partials + (size_t)rows * NSTAT;
-        e = storage == 2
-                ? (d2 ? launch_refine16_d2q9(diag, check, pf, grid, fgrid,
-                                             h->stream)
-                      : launch_refine16_d3q27(diag, check, pf, grid, fgrid,
-                                              h->stream))
-                : (d2 ? launch_refine_d2q9(diag, check, pf, grid, fgrid,
-                                           h->stream)
-                      : launch_refine_d3q27(diag, check, pf, grid, fgrid,
-                                            h->stream));
+        e = storage == 2 ? launch_refine16_d3q27(diag, check, pf, grid, fgrid,
+                                                 h->stream)
+                         : launch_refine_d3q27(diag, check, pf, grid, fgrid,
+                                               h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "second stage launch");
         rows += fgrid;
       }

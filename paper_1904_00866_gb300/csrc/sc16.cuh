@@ -81,19 +81,26 @@ __global__ void __launch_bounds__(kSc32Threads, 2)
       const unsigned sh = ((upper >> i) & 1u) << 4;
       return h16_dev<L>((unsigned short)(w >> sh), i);
     };
+    auto out = [&](int i, float v) {
+      reinterpret_cast<unsigned short*>(p.out_pop[i])[node] =
+          h16_bits<L>(v, i);
+    };
     unsigned st = kNodeDone;
     float ap = 0.0f;
     if (node < (unsigned)p.n)
       st = sc32_node_in<L, true, DIAG, CHECK>(
           in, rho0f, p.rho0, beta, 0.0f, nullptr,
           p.alpha_map ? p.alpha_map + node : nullptr, acc,
-          [&](int i, float v) {
-            reinterpret_cast<unsigned short*>(p.out_pop[i])[node] =
-                h16_bits<L>(v, i);
-          },
-          p.exact ? &ap : nullptr);
-    if (p.exact)
-      defer_undecided<L>(p, &s_refine, st == kNodeRefine, in, node, ap);
+          out, p.exact ? &ap : nullptr);
+    // D2Q9: the second stage here, as in k_sc32
+    if constexpr (Q == 9) {
+      if (p.exact)
+        st = refine_inline<L, true, DIAG, CHECK>(p, in, node, st, ap, acc,
+                                                 out);
+    } else {
+      if (p.exact)
+        defer_undecided<L>(p, &s_refine, st == kNodeRefine, in, node, ap);
+    }
     defer_nodes(&p.far_count[p.parity], p.far_queue, p.far_cap, p.err_flags,
                 node, st == kNodeFar ? kNodeFar : kNodeDone);
   }
