@@ -65,6 +65,7 @@ __device__ __forceinline__ int refine_deferred(const StepParams& p,
 template <class L, class S, int DIAG, int CHECK>
 __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
                                                          int blocks) {
+  chain_begin();
   constexpr int Q = L::Q;
   __shared__ unsigned pre[kMaxRefineBlocks + 1];
   block_prefix(p.refine_counts, blocks, pre);
@@ -192,6 +193,7 @@ __device__ __forceinline__ unsigned open_warps(unsigned count,
 
 template <class L, class S, int DIAG, int CHECK>
 __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
+  chain_begin();
   constexpr int Q = L::Q;
   const unsigned count = min(p.far_count[p.parity], p.far_cap);
   const unsigned open_count = min(p.far_count[2 + p.parity], p.far_cap);

@@ -12,6 +12,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 
 namespace elbm {
@@ -32,17 +33,33 @@ static cudaError_t set_smem_limit(Kernel k, int bytes,
   return e;
 }
 
+// Blocks of a kernel one device holds at a time, asked for once per device
+// and instantiation (the queries cost the host more than the launch).
+struct ResidentBlocks {
+  std::atomic<int> on[64];
+};
 template <class Kernel>
-static int occupancy_grid(Kernel k, int block, long long threads_needed) {
-  int dev = 0, sms = 0, per_sm = 0;
+static int resident_blocks(Kernel k, int block, int smem, ResidentBlocks& c) {
+  int dev = 0;
   cudaGetDevice(&dev);
+  const bool kept = dev >= 0 && dev < 64;
+  int g = kept ? c.on[dev].load(std::memory_order_relaxed) : 0;
+  if (g > 0) return g;
+  int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
   if (per_sm < 1) per_sm = 1;
   if (per_sm > 2048 / block) per_sm = 2048 / block;   // partials rows bound
-  long long g = (long long)sms * per_sm;
-  const long long need = (threads_needed + block - 1) / block;
-  if (need < g) g = need;
+  g = sms * per_sm;
+  if (kept && g > 0) c.on[dev].store(g, std::memory_order_relaxed);
+  return g;
+}
+// The grid of a persistent kernel: resident blocks, capped by the work.
+template <class Kernel>
+static int occupancy_grid(Kernel k, int block, int smem, long long blocks,
+                          ResidentBlocks& c) {
+  const long long g =
+      std::min<long long>(resident_blocks(k, block, smem, c), blocks);
   return g < 1 ? 1 : (int)g;
 }
 
@@ -50,7 +67,10 @@ template <class L, class T, int MODE, int DIAG, int CHECK>
 static cudaError_t launch_one(const StepParams& p, int grid, int block,
                               cudaStream_t s, int* grid_used) {
   auto k = k_stream_collide<L, T, MODE, DIAG, CHECK>;
-  if (grid <= 0) grid = occupancy_grid(k, block, p.tiles * 32);
+  static ResidentBlocks resident;
+  if (grid <= 0)
+    grid = occupancy_grid(k, block, 0, (p.tiles * 32 + block - 1) / block,
+                          resident);
   if (grid_used) *grid_used = grid;
   k<<<grid, block, 0, s>>>(p);
   count_launch();
@@ -65,17 +85,18 @@ template <class L, class T, int MODE, int DIAG>
 static cudaError_t launch_sc64(const StepParams& p, cudaStream_t s,
                                int* grid_used) {
   auto k = k_sc64<L, T, MODE, DIAG>;
+  static ResidentBlocks resident;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long warps = (p.n + 31) / 32;
   const int block = warps <= 4LL * sms ? 32 : 128;
-  const int grid = block == 32 ? (int)warps
-                               : occupancy_grid(k, block, p.n);
+  const int grid =
+      block == 32 ? (int)warps
+                  : occupancy_grid(k, block, 0, (p.n + block - 1) / block,
+                                   resident);
   if (grid_used) *grid_used = grid;
-  k<<<grid, block, 0, s>>>(p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_chained(k, grid, block, 0, s, p.chained, p);
 }
 
 template <class L, class T, int MODE>
@@ -115,23 +136,12 @@ static cudaError_t launch_sc32_one(const StepParams& p, int grid,
   static std::atomic<unsigned long long> configured{0};   // per instantiation
   const cudaError_t se = set_smem_limit(k, smem, configured);
   if (se != cudaSuccess) return se;
-  if (grid <= 0) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kSc32Threads,
-                                                  smem);
-    if (per_sm < 1) per_sm = 1;
-    if (per_sm > 2048 / kSc32Threads) per_sm = 2048 / kSc32Threads;
-    long long g = (long long)sms * per_sm;
-    const long long tiles = (p.n + kSc32Threads - 1) / kSc32Threads;
-    if (tiles < g) g = tiles;
-    grid = g < 1 ? 1 : (int)g;
-  }
+  static ResidentBlocks resident;
+  if (grid <= 0)
+    grid = occupancy_grid(k, kSc32Threads, smem,
+                          (p.n + kSc32Threads - 1) / kSc32Threads, resident);
   if (grid_used) *grid_used = grid;
-  k<<<grid, kSc32Threads, smem, s>>>(p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_chained(k, grid, kSc32Threads, smem, s, p.chained, p);
 }
 
 template <class L, bool SHIFTED>
@@ -246,23 +256,12 @@ static cudaError_t launch_sc16_one(const StepParams& p, int grid,
   static std::atomic<unsigned long long> configured{0};   // per instantiation
   const cudaError_t se = set_smem_limit(k, smem, configured);
   if (se != cudaSuccess) return se;
-  if (grid <= 0) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kSc32Threads,
-                                                  smem);
-    if (per_sm < 1) per_sm = 1;
-    if (per_sm > 2048 / kSc32Threads) per_sm = 2048 / kSc32Threads;
-    long long g = (long long)sms * per_sm;
-    const long long tiles = (p.n + kSc32Threads - 1) / kSc32Threads;
-    if (tiles < g) g = tiles;
-    grid = g < 1 ? 1 : (int)g;
-  }
+  static ResidentBlocks resident;
+  if (grid <= 0)
+    grid = occupancy_grid(k, kSc32Threads, smem,
+                          (p.n + kSc32Threads - 1) / kSc32Threads, resident);
   if (grid_used) *grid_used = grid;
-  k<<<grid, kSc32Threads, smem, s>>>(p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_chained(k, grid, kSc32Threads, smem, s, p.chained, p);
 }
 
 template <class L>
@@ -281,14 +280,9 @@ static cudaError_t launch_far_lattice(int diag, int check,
                                       const StepParams& p, int grid,
                                       cudaStream_t s) {
   if (grid <= 0) grid = 152;
-  if (check)
-    k_far_fixup<L, S, 1, 1><<<grid, 256, 0, s>>>(p);
-  else if (diag)
-    k_far_fixup<L, S, 1, 0><<<grid, 256, 0, s>>>(p);
-  else
-    k_far_fixup<L, S, 0, 0><<<grid, 256, 0, s>>>(p);
-  count_launch();
-  return cudaGetLastError();
+  auto k = check ? k_far_fixup<L, S, 1, 1>
+                 : (diag ? k_far_fixup<L, S, 1, 0> : k_far_fixup<L, S, 0, 0>);
+  return launch_chained(k, grid, 256, 0, s, p.chained, p);
 }
 
 // Second stage of the undecided nodes a stream-collide launch of `blocks`
@@ -299,14 +293,9 @@ static cudaError_t launch_refine_lattice(int diag, int check,
                                          int grid, cudaStream_t s) {
   if (blocks > kMaxRefineBlocks) return cudaErrorInvalidValue;
   if (grid <= 0) grid = 152;
-  if (check)
-    k_refine_stage<L, S, 1, 1><<<grid, 256, 0, s>>>(p, blocks);
-  else if (diag)
-    k_refine_stage<L, S, 1, 0><<<grid, 256, 0, s>>>(p, blocks);
-  else
-    k_refine_stage<L, S, 0, 0><<<grid, 256, 0, s>>>(p, blocks);
-  count_launch();
-  return cudaGetLastError();
+  auto k = check ? k_refine_stage<L, S, 1, 1>
+                 : (diag ? k_refine_stage<L, S, 1, 0> : k_refine_stage<L, S, 0, 0>);
+  return launch_chained(k, grid, 256, 0, s, p.chained, p, blocks);
 }
 
 }  // namespace elbm

@@ -26,8 +26,8 @@ void count_launches(long long n) {
 }
 
 // Sum the partial rows of one step in a fixed order.
-__global__ void k_finish(const double* __restrict__ partials, int rows,
-                         double* __restrict__ out) {
+__global__ void k_finish(const double* partials, int rows, double* out) {
+  chain_begin();
   const int k = blockIdx.x;  // slot
   __shared__ double sm[256];
   double v = k < S_NSUM ? 0.0 : (k == S_AMIN ? INFINITY : -INFINITY);
@@ -67,10 +67,9 @@ __global__ void k_partial_sum(const double* __restrict__ x, long long n,
 }
 
 cudaError_t launch_finish(const double* partials, int rows, double* out,
-                          cudaStream_t s) {
-  k_finish<<<NSTAT, 256, 0, s>>>(partials, rows, out);
-  count_launch();
-  return cudaGetLastError();
+                          int chained, cudaStream_t s) {
+  return launch_chained(k_finish, NSTAT, 256, 0, s, chained, partials, rows,
+                        out);
 }
 
 void stats_from_slots(const double* s, double rho0, long long n,
@@ -626,6 +625,11 @@ elbm_status elbm_step(elbm_handle* h, long long nsteps, elbm_alpha_mode mode) {
     }
     p.alpha_map = amap ? h->alpha_map : nullptr;
     p.parity = (int)(n & 1);
+    // the first kernel follows the counters' clear; events between the
+    // kernels (profiling) take the plain order
+    const int chained =
+        !h->profiling && chain_pays((double)p.ps * h->q * esz);
+    p.chained = chained && s > 0;
     int grid = 0;
     cudaError_t e;
     const bool fp32_formula = storage != 0 && mode == ELBM_ALPHA_FORMULA;
@@ -667,6 +671,7 @@ elbm_status elbm_step(elbm_handle* h, long long nsteps, elbm_alpha_mode mode) {
     int rows = grid;
     if (fp32_formula) {
       StepParams pf = p;
+      pf.chained = chained;
       // the second stage runs 2 blocks per SM and the fixup one (their
       // register budgets), so a larger grid only adds waves of blocks with
       // nothing to do
@@ -693,7 +698,7 @@ elbm_status elbm_step(elbm_handle* h, long long nsteps, elbm_alpha_mode mode) {
       rows += xgrid;
     }
     if (diag) {
-      launch_finish(h->partials, rows, h->stats_dev, h->stream);
+      launch_finish(h->partials, rows, h->stats_dev, chained, h->stream);
       h->stats_valid = true;
       h->stats_step = n;
       h->stats_checked = check;

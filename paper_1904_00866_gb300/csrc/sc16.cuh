@@ -46,6 +46,7 @@ __device__ __forceinline__ unsigned issue_tile16(const StepParams& p,
 template <class L, int DIAG, int CHECK>
 __global__ void __launch_bounds__(kSc32Threads, 2)
     k_sc16(const StepParams p) {
+  chain_begin();
   constexpr int Q = L::Q;
   extern __shared__ unsigned smem_w[];   // [2][Q][256] words
   const unsigned ntiles = (unsigned)((p.n + kSc32Threads - 1) / kSc32Threads);

@@ -538,6 +538,7 @@ __device__ __forceinline__ unsigned refine_inline(const StepParams& p, In in,
 template <class L, bool SHIFTED, int DIAG, int CHECK>
 __global__ void __launch_bounds__(kSc32Threads, L::Q == 9 && !CHECK ? 3 : 2)
     k_sc32(const StepParams p) {
+  chain_begin();
   constexpr int Q = L::Q;
   extern __shared__ float smem[];   // [2][Q][256]
   __shared__ unsigned s_refine;     // this block's undecided-node entries

@@ -98,6 +98,7 @@ __device__ __noinline__ Collided64 far64_node(const StepParams& p,
 
 template <class L, class T, int MODE, int DIAG>
 __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
+  chain_begin();
   constexpr int Q = L::Q;
   const T* __restrict__ fin = static_cast<const T*>(p.f_in);
   T* __restrict__ fout = static_cast<T*>(p.f_out);

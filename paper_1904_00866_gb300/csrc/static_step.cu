@@ -158,13 +158,14 @@ extern "C" elbm_status elbm_step_static(
   if (e != cudaSuccess) return fail(ELBM_ECUDA, cudaGetErrorString(e));
   const int fgrid = grid < 152 ? grid : 152;   // grid + fgrid <= rows (above)
   StepParams pf = p;
+  pf.chained = chain_pays((double)n * q * sizeof(float));
   pf.partials = partials + (size_t)grid * NSTAT;
   e = lattice == ELBM_D2Q9 ? launch_far_d2q9(diag, 0, pf, fgrid, stream)
                            : launch_far_d3q27(diag, 0, pf, fgrid, stream);
   if (e != cudaSuccess) return fail(ELBM_ECUDA, cudaGetErrorString(e));
   if (!diag) return ELBM_OK;
 
-  e = launch_finish(partials, grid + fgrid, stats, stream);
+  e = launch_finish(partials, grid + fgrid, stats, pf.chained, stream);
   if (e != cudaSuccess) return fail(ELBM_ECUDA, cudaGetErrorString(e));
   double slots[NSTAT];
   unsigned flags = 0;

@@ -9,6 +9,16 @@
 
 namespace elbm {
 
+// First statement of every kernel that launch_chained launches: lets the
+// next kernel of the chain be scheduled as soon as every block of this one
+// runs, and waits until the previous kernel has completed (no wait when the
+// launch was not chained).  All threads call it before any access to memory
+// another kernel writes, so completion is transitive along the chain.
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Partial slots.  Slots [0, S_NSUM) are sums, the rest min / max.
 enum {
   S_DRHO = 0,   // sum (rho - rho0)

@@ -81,6 +81,7 @@ struct StepParams {
   float corr_rho;         // unshifted: sum_i fl(W_i rho0) - rho0
   float corr[27];         // unshifted: W_i rho0 - fl(W_i rho0)
   int secant_iters;
+  int chained;            // host: launched right after a kernel of this call
   unsigned* far_count;    // [4] by step parity: [0..1] deferred nodes (from
                           // the queue's bottom), [2..3] nodes the second
                           // stage left open (from its top)
