@@ -493,11 +493,26 @@ static elbm_status autotune(elbm_batch* b) {
       elbm_status st = upload_tables(b);
       if (st) return st;
       const int grid = sms * bps;
-      run_steps(b, 1, 0, grid);   // warm-up (dry: steps_left = 1, step 0)
-      cudaEventRecord(e0, b->stream);
-      for (int r = 0; r < 3; ++r) run_steps(b, 1, 0, grid);
-      cudaEventRecord(e1, b->stream);
-      cudaError_t ce = cudaEventSynchronize(e1);
+      // Only the stream-collide kernel's shape is chosen, so only it is
+      // timed, and without the undecided-node records: a batch is tuned
+      // right after its members' initialisation, when nearly every node is
+      // undecided, and the time of a whole step (mostly its fixup, ~10x a
+      // developed step's) left the choice to chance (12 members of the
+      // server's mix: 115 us per step with the 128-thread shape it took in
+      // two processes of four, 102 with the other).
+      BatchParams bp = batch_params(b);
+      bp.exact = 0;
+      cudaError_t ce = cudaSuccess;
+      for (int r = 0; r < 4 && ce == cudaSuccess; ++r) {
+        if (r == 1) cudaEventRecord(e0, b->stream);   // r = 0: warm-up
+        ce = cudaMemsetAsync(b->d_far_count, 0, 4 * sizeof(unsigned),
+                             b->stream);
+        if (ce == cudaSuccess) ce = launch_batch(tb, 0, bp, grid, b->stream);
+      }
+      if (ce == cudaSuccess) {
+        cudaEventRecord(e1, b->stream);
+        ce = cudaEventSynchronize(e1);
+      }
       if (ce != cudaSuccess) return bfail(b, ELBM_ECUDA, cudaGetErrorString(ce));
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
