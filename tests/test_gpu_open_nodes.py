@@ -6,8 +6,9 @@ around a warp, a block and the fixup's list lengths, right after
 initialisation (n is rounding noise) and some steps later.
 
 Reference: Eqs. (8)-(9) of the stored state by the power series of Delta H
-in extended precision.  Where |Delta H(2)| > 2^-44 M_2 (M_2 = sum f x^2) the
-branch is the reference's: every evaluation's error is below 2^-45 M_2.
+in FP64 (n off by less than 20 u f, so Delta H(2) by 20 u M_2, u = 2^-53,
+M_2 = sum f x^2).  Where |Delta H(2)| > 2^-44 M_2 the branch is the
+reference's: the error of every evaluation in the library is below 2^-45 M_2.
 alpha there is within 2^-16 of Eq. (9) (the width the FP32 stages certify)
 plus one FP32 rounding.  Populations follow from the alpha taken within the
 FP32 relaxation (2e-6 |f|), plus for binary16 storage one rounding of the
@@ -37,9 +38,8 @@ def elbm():
 
 def _reference(f, c, w, d):
     """n = f^eq - f, Delta H(2), the Eq. (9) chord and M_2 of every node."""
-    f = f.astype(np.longdouble)
     rho = f.sum(0)
-    feq = rho * w.reshape((-1,) + (1,) * 3).astype(np.longdouble)
+    feq = rho * w.reshape((-1,) + (1,) * 3)
     for a in range(d):
         ca = c[:, a].reshape((-1,) + (1,) * 3)
         u = (ca * f).sum(0) / rho
@@ -89,7 +89,7 @@ def test_open_nodes(elbm, lat, n, warm, dtype):
     assert np.abs(a - chord)[sure].max(initial=0) <= 2.0 ** -16 + 2.0 ** -22
     beta = 1 / (6 * nu + 1)
     for i in range(len(f)):
-        want = (f[i] + a * beta * ne[i]).astype(np.float64)
+        want = f[i] + a * beta * ne[i]
         tol = 2e-6 * np.abs(want)
         if dtype == "fp16_shifted":
             tol += 2.0 ** -10 * np.abs(want - w[i] * g.rho0) + 2.0 ** -24
