@@ -172,12 +172,12 @@ __device__ __forceinline__ void relax_store32(const N32<L>& r, float d0,
   const float ab = r.alpha * beta;
   projection<L>(
       r,
-      [&](float wt) {
-        const float nv = fmaf(ab, r.n0 - wt, d0);
+      [&](float m) {
+        const float nv = fmaf(ab, m, d0);
         out(0, SHIFTED ? nv : nv + L::wf(0) * rho0f);
       },
-      [&](int k, float2 wt) {
-        float2 nv = fma2(f2(ab), sub2(r.n2[k], wt), dd[k]);
+      [&](int k, float2 m) {
+        float2 nv = fma2(f2(ab), m, dd[k]);
         if (!SHIFTED) nv = add2(nv, f2(L::wf(2 * k + 1) * rho0f));
         out(2 * k + 1, nv.x);
         out(2 * k + 2, nv.y);
@@ -197,8 +197,7 @@ __device__ __forceinline__ void relax_update32(const N32<L>& r, float ap,
   const float abp = ap * beta, abe = ae * beta;
   projection<L>(
       r,
-      [&](float wt) {
-        const float m = r.n0 - wt;
+      [&](float m) {
         float vp = fmaf(abp, m, d0), ve = fmaf(abe, m, d0);
         if (!SHIFTED) {
           vp += L::wf(0) * rho0f;
@@ -206,8 +205,7 @@ __device__ __forceinline__ void relax_update32(const N32<L>& r, float ap,
         }
         if (ve != vp) out(0, ve);
       },
-      [&](int k, float2 wt) {
-        const float2 m = sub2(r.n2[k], wt);
+      [&](int k, float2 m) {
         float2 vp = fma2(f2(abp), m, dd[k]), ve = fma2(f2(abe), m, dd[k]);
         if (!SHIFTED) {
           vp = add2(vp, f2(L::wf(2 * k + 1) * rho0f));
