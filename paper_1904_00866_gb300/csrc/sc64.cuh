@@ -132,9 +132,7 @@ __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
       unsigned flags = 0;
       int iters = 0;
       double alpha = 2.0;
-      if (se.rest)
-        flags = NF_DEGENERATE;
-      else if (MODE == MODE_ROOT)
+      if (MODE == MODE_ROOT)
         alpha = alpha_root_near(nd, se, flags, iters);
       else if (MODE == MODE_SECANT)
         alpha = alpha_secant_near(se, p.secant_iters, flags, iters);

@@ -29,7 +29,8 @@
 // instructions issue on the FP64 pipe.
 //
 // Nodes outside the range (|x_i| > 1/32, |u_a| >= 1/4, f_i below 2^-12 of
-// the largest, invalid states) report false and take the logarithm path.
+// the largest, every |n_i| below 2^-42 of it, invalid states) report false
+// and take the logarithm path.
 #pragma once
 #include "df32.cuh"
 #include "fp16_storage.cuh"
@@ -40,6 +41,14 @@ namespace elbm {
 
 constexpr int kSeriesTop = 14;             // last moment of the series
 constexpr float kSeriesXMax = 0.03125f;    // largest |x_i| it takes
+// Exponent of max |n_i| over that of max f_i below which f^eq == f to within
+// the rounding of either form: whether a node counts as degenerate, and the
+// sign of Delta H(2) ~ x M_2 / 3 against the logarithm form's 1.1e-14 M_2,
+// are then decided by rounding, and the logarithm form (max |n_i| up to 27
+// times 20 ulp of the largest f_i at a node it finds degenerate) keeps that
+// decision.  Only states at equilibrium get there: the first step after
+// initialisation, a fluid at rest.
+constexpr int kSeriesNMin = -42;
 
 // (double)v for normal or zero v, by shifting the exponent and mantissa
 __device__ __forceinline__ double f2d(float v) {
@@ -110,7 +119,6 @@ struct Series64 {
   DF<float> m[7];               // k = 2..6
   float t[kSeriesTop + 1];      // k = 7..kSeriesTop
   int e_n, e_d;                 // en = 2^e_n, d = 2^e_d
-  bool rest;                    // f^eq = f to FP64 rounding
 };
 
 // 1 / y for normal y: the SFU's value (relative error below 2^-20) and one
@@ -254,9 +262,7 @@ __device__ __forceinline__ bool near64_prepare(Near64<L>& s, Series64& r) {
   const int nexp = (nmax & 0x7ff00000) + (6 << 20);
   r.e_n = (nexp >> 20) - 1023;
   r.e_d = (nexp - rexp) >> 20;
-  // |n_i| < 2^-59 rho: within the last bits of the smallest populations
-  r.rest = r.e_d < -54;
-  if (r.rest) return true;
+  if (r.e_d < kSeriesNMin + 3) return false;
   const float d = __int_as_float((127 + r.e_d) << 23);
 
   const int adjn = nexp - (127 << 20), adjf = rexp - (127 << 20);
@@ -389,13 +395,13 @@ __device__ __forceinline__ double alpha_formula_near(const Series64& r,
 // (u = 2^-53; 27 terms f phi(2 x) of at most 2 f x^2, the products f x L,
 // and x off by 20 u), the series' by less than 20 u M_2, so a value beyond
 // 2^-45 M_2 has the same sign in both, and the two alphas differ by less
-// than 1e-13.  False: out of the series' range, at rest, or within that
-// distance of zero -- the logarithm form decides.
+// than 1e-13.  False: out of the series' range or within that distance of
+// zero -- the logarithm form decides.
 template <class L>
 __device__ __forceinline__ bool near64_formula(Near64<L>& s, double& alpha,
                                                unsigned& flags) {
   Series64 r;
-  if (!near64_prepare(s, r) || r.rest) return false;
+  if (!near64_prepare(s, r)) return false;
   const float d = __int_as_float((127 + r.e_d) << 23);
   const DF<float> b2 = series_sum<3, true>(r, d);
   if (!(fabsf(b2.hi) * d > 2.842170943040401e-14f * r.m[2].hi)) return false;

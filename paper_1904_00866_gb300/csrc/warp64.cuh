@@ -204,7 +204,7 @@ __device__ __forceinline__ bool near64_warp(const LanePop& lp, int lane,
       kAll, lp.on ? __double2hiint(n) & 0x7fffffff : 0);
   const int nexp = (nmax & 0x7ff00000) + (6 << 20);
   const int e_d = (nexp - rexp) >> 20;
-  if (e_d < -54) return false;   // at rest
+  if (e_d < kSeriesNMin + 3) return false;
   const float d = __int_as_float((127 + e_d) << 23);
   // this lane's x (in units of d) and series terms; idle lanes add zeros
   const DF<float> zero = {0.0f, 0.0f}, one = {1.0f, 0.0f};
