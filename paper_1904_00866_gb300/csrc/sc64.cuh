@@ -128,7 +128,8 @@ __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
       }
     }
     Series64 se;
-    if (near64_prepare(nd, se)) {
+    if (near64_prepare(
+            nd, se, sizeof(T) == 8 ? kSeriesXMax : kSeriesXMaxRounded)) {
       unsigned flags = 0;
       int iters = 0;
       double alpha = 2.0;

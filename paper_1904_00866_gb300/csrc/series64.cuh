@@ -1,5 +1,6 @@
-// FP64 collision of a node near equilibrium (max |x_i| <= 1/32) without
-// logarithms, for FP64 storage and the ROOT / SECANT modes.
+// FP64 collision of a node near equilibrium (max |x_i| <= 1/48, or 1/32
+// where alpha is rounded to FP32) without logarithms, for FP64 storage and
+// the ROOT / SECANT modes.
 //
 // What bounds it: GB300 issues one FP64 warp instruction per 64 cycles on
 // each SM sub-partition, against one FP32 or integer instruction per cycle.
@@ -18,17 +19,21 @@
 // alpha = 2, so Delta H(2) is formed from its own leading term M_3 instead
 // of as the difference of two O(x^2) sums: with x_i and M_2..M_6 in
 // double-float (relative error ~2^-44) and M_7..M_14 in FP32, Delta H(2) is
-// off by ~1e-13 x^3 rho, less than the ~1e-16 x^2 rho of the logarithm form
-// for every x <= 1/1000 and within a few times it at 1/32, and alpha beta n
-// is off by less than 2e-13 x^2 f, below half an ulp of f.  The series is
-// cut after k = 14: 2^15 x^15 / 210 < 4e-18 x^2 at x = 1/32.
+// off by ~1e-13 x^3 rho plus 2e-7 x^7 rho, against ~1e-16 x^2 rho of the
+// logarithm form.  The range ends where the second term reaches that.
+// Measured against 160 bits over max |x| = 1e-11 .. 0.024, 320 states per
+// lattice: alpha off by at most 8.5e-16 (D2Q9) and 7.7e-16 (D3Q27), the
+// logarithm form's by 1.8e-15 and 3.0e-15; the new populations by 1.1e-15
+// and 1.3e-15 of f, the logarithm form's by 1.1e-15 and 1.8e-15.  At 1/32
+// alpha would be off by 1.1e-14.  The series is cut after k = 14:
+// 2^15 x^15 / 210 < 3e-20 x^2 at x = 1/48.
 //
 // Numbers are scaled by powers of two before they become FP32 (n_i by that
 // of max |n_i|, f_i by that of max f_i), so nothing under- or overflows.
 // Conversions between FP64 and FP32 are integer shifts: the conversion
 // instructions issue on the FP64 pipe.
 //
-// Nodes outside the range (|x_i| > 1/32, |u_a| >= 1/4, f_i below 2^-12 of
+// Nodes outside the range (|x_i| too large, |u_a| >= 1/4, f_i below 2^-12 of
 // the largest, every |n_i| below 2^-42 of it, invalid states) report false
 // and take the logarithm path.
 #pragma once
@@ -40,7 +45,12 @@
 namespace elbm {
 
 constexpr int kSeriesTop = 14;             // last moment of the series
-constexpr float kSeriesXMax = 0.03125f;    // largest |x_i| it takes
+// Largest |x_i| it takes.  Where alpha is rounded to FP32 afterwards (FP32 /
+// FP16 storage) an error of 1e-14 does not matter and the range is wider, as
+// the fixup's open nodes between the two would cost a logarithm form each
+// (189 x 107 x 83, 20 steps: 2.95 ms with 1/48, 2.85 with 1/32).
+constexpr float kSeriesXMax = 1.0f / 48.0f;
+constexpr float kSeriesXMaxRounded = 1.0f / 32.0f;
 // Exponent of max |n_i| over that of max f_i below which f^eq == f to within
 // the rounding of either form: whether a node counts as degenerate, and the
 // sign of Delta H(2) ~ x M_2 / 3 against the logarithm form's 1.1e-14 M_2,
@@ -160,9 +170,10 @@ struct Near64 {
 };
 
 // Moments, n_i and the scaled x moments of a node whose f[] is filled.
-// False: the node is outside the series' range.
+// False: the node is outside the series' range, max |x_i| <= xmax.
 template <class L>
-__device__ __forceinline__ bool near64_prepare(Near64<L>& s, Series64& r) {
+__device__ __forceinline__ bool near64_prepare(Near64<L>& s, Series64& r,
+                                               float xmax) {
   constexpr int Z = L::D == 3 ? 1 : 0;
   int fmin = 0x7fffffff, fmax = (int)0x80000000;
 #pragma unroll
@@ -179,8 +190,7 @@ __device__ __forceinline__ bool near64_prepare(Near64<L>& s, Series64& r) {
   // Mass and momentum in 64-bit integers: exact, and off the FP64 pipe (49
   // additions for D3Q27).  Within the series' range f_0 >= 0.2 rho, so rho
   // stays below 2^4 of the largest f_i's power of two; a node for which it
-  // does not overflows, and its f^eq then differs from f far beyond
-  // kSeriesXMax.
+  // does not overflows, and its f^eq then differs from f far beyond xmax.
   const int top = rexp + (1 << 20) + 0xfffff;
   long long jx = 0, jy = 0;
   long long sy[3];
@@ -327,7 +337,7 @@ __device__ __forceinline__ bool near64_prepare(Near64<L>& s, Series64& r) {
       tt[q] = add_(tt[q], w);
     }
   }
-  if (!(fmaxf(xm.x, xm.y) * d <= kSeriesXMax)) return false;
+  if (!(fmaxf(xm.x, xm.y) * d <= xmax)) return false;
   auto fold = [](const DF<float2>& m) {
     return df_add(fast_two_sum(m.hi.x, m.lo.x), fast_two_sum(m.hi.y, m.lo.y));
   };
@@ -401,7 +411,7 @@ template <class L>
 __device__ __forceinline__ bool near64_formula(Near64<L>& s, double& alpha,
                                                unsigned& flags) {
   Series64 r;
-  if (!near64_prepare(s, r)) return false;
+  if (!near64_prepare(s, r, kSeriesXMaxRounded)) return false;
   const float d = __int_as_float((127 + r.e_d) << 23);
   const DF<float> b2 = series_sum<3, true>(r, d);
   if (!(fabsf(b2.hi) * d > 2.842170943040401e-14f * r.m[2].hi)) return false;

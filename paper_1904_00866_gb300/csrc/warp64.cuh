@@ -212,7 +212,7 @@ __device__ __forceinline__ bool near64_warp(const LanePop& lp, int lane,
   const DF<float> ff = lp.on ? split_df(f, rexp - (127 << 20)) : one;
   const DF<float> x = df_div(nn, ff);
   const int xm = __reduce_max_sync(kAll, __float_as_int(fabsf(x.hi)));
-  if (!(__int_as_float(xm) * d <= kSeriesXMax)) return false;
+  if (!(__int_as_float(xm) * d <= kSeriesXMaxRounded)) return false;
   const DF<float> y = {x.hi * d, x.lo * d};   // exact
   float t2 = 0.0f, t1 = 0.0f;
 #pragma unroll
