@@ -49,8 +49,8 @@ __device__ __forceinline__ void pull_sources(const StepParams& p,
 template <class L, class T, int MODE>
 __device__ __noinline__ Collided64 far64_node(const StepParams& p,
                                               unsigned node) {
-  const T* __restrict__ fin = static_cast<const T*>(p.f_in);
-  T* __restrict__ fout = static_cast<T*>(p.f_out);
+  const T* fin = static_cast<const T*>(p.f_in);
+  T* fout = static_cast<T*>(p.f_out);
   int x, y, z;
   pull_sources<L>(p, node, x, y, z);
   Node64<L> nd;
@@ -100,8 +100,8 @@ template <class L, class T, int MODE, int DIAG>
 __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
   chain_begin();
   constexpr int Q = L::Q;
-  const T* __restrict__ fin = static_cast<const T*>(p.f_in);
-  T* __restrict__ fout = static_cast<T*>(p.f_out);
+  const T* fin = static_cast<const T*>(p.f_in);
+  T* fout = static_cast<T*>(p.f_out);
   Acc acc;
   if (DIAG) acc.init();
   for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < p.n;

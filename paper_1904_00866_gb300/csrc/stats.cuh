@@ -14,6 +14,10 @@ namespace elbm {
 // runs, and waits until the previous kernel has completed (no wait when the
 // launch was not chained).  All threads call it before any access to memory
 // another kernel writes, so completion is transitive along the chain.
+// A chained grid may be resident while its predecessor still writes, so
+// nothing the predecessor writes is constant for the kernel's duration: no
+// __restrict__ and no read-only load on such data, which would let loads
+// take the non-coherent path or move above the wait.
 __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
