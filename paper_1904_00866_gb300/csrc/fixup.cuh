@@ -37,8 +37,8 @@ __device__ __forceinline__ int refine_deferred(const StepParams& p,
       p.alpha_map ? p.alpha_map + node : nullptr, ap, out,
       [&](const N32<L>& r) {
         if (!DIAG) return;
-        if constexpr (std::is_same<A, Acc32>::value) {
-          diag32<L, SHIFTED, CHECK>(r, in, p.rho0, acc);
+        if constexpr (!std::is_same<A, Acc>::value) {
+          diag32<L, SHIFTED, CHECK, true>(r, in, p.rho0, acc);
         } else {
           const double j[3] = {r.j[0], r.j[1], r.j[2]};
           acc.add_moments((double)r.drho, j, (double)r.rho);
@@ -72,10 +72,7 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
   const unsigned total = pre[blocks];
   const unsigned seg = p.refine_cap / (unsigned)blocks;
   const bool shifted = sizeof(S) == 2 || !p.unshifted;
-  // compensated FP32 sums, as in the stream-collide kernels: FP64 ones (with
-  // their division) take ~25 instructions of 64 cycles per node (32^3 with
-  // statistics on every step: 41 -> 36 us per step)
-  Acc32 acc;
+  Acc32T<Sum2> acc;
   acc.init();
   for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < total;
        k += gridDim.x * blockDim.x) {

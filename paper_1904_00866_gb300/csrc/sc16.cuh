@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kSc32Threads, 2)
   const unsigned ntiles = (unsigned)((p.n + kSc32Threads - 1) / kSc32Threads);
   const float rho0f = p.rho0f;
   const float beta = p.betaf;
-  Acc32 acc;
+  AccSc<L> acc;
   if (DIAG) acc.init();
   __shared__ unsigned s_refine;     // this block's undecided-node entries
   refine_block_begin(&s_refine);

@@ -12,6 +12,8 @@
 #pragma once
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "node_fp32.cuh"
 #include "stream_collide.cuh"
 
@@ -48,8 +50,31 @@ struct KSum {
   }
 };
 
-struct Acc32 {
-  KSum drho, j0, j1, j2, ke, asum;
+// The same with the additions' roundings summed on their own (Sum2 of Ogita,
+// Rump & Oishi, "Accurate sum and dot product", 2005): as if summed in twice
+// the precision, off by about n 2^-48 sum |v|, where Kahan's sum, which rounds
+// v - c to FP32 at each term, keeps up to 2^-24 of a term.  For the sums that
+// second-stage nodes enter, in place of FP64 ones on the FP64 pipe.
+struct Sum2 {
+  float s, c;
+  __device__ __forceinline__ void init() { s = c = 0.0f; }
+  __device__ __forceinline__ void add(float v) {
+    const DF<float> t = two_sum(s, v);
+    s = t.hi;
+    c = add_(c, t.lo);
+  }
+  __device__ __forceinline__ void add(const DF<float>& v) {
+    add(v.hi);
+    c = add_(c, v.lo);
+  }
+  __device__ __forceinline__ double value() const {
+    return (double)s + (double)c;
+  }
+};
+
+template <class S>
+struct Acc32T {
+  S drho, j0, j1, j2, ke, asum;
   float amin, amax;
   unsigned nodes, acc2, formula, band, degen;
   double h, adev;
@@ -63,11 +88,16 @@ struct Acc32 {
     viol = mismatch = 0u;
   }
 };
+using Acc32 = Acc32T<KSum>;
+// Accumulators of a stream-collide kernel: D2Q9 kernels run the second stage
+// too.  (Sum2 costs the D3Q27 kernels 2 % of a step with statistics.)
+template <class L>
+using AccSc = Acc32T<typename std::conditional<L::Q == 9, Sum2, KSum>::type>;
 
 // Block reduction of the per-thread FP32 accumulators into one partials
 // row (FP64 slots).
-__device__ __forceinline__ void store_acc32(const Acc32& acc,
-                                            double* partials) {
+template <class A>
+__device__ __forceinline__ void store_acc32(const A& acc, double* partials) {
   Acc a;
   a.init();
   a.drho = acc.drho.value();
@@ -230,17 +260,27 @@ __device__ __forceinline__ Check64 check32(In in, double rho0, float alpha,
   return node64_check(nd, (double)alpha);
 }
 
-// Statistics of one collided node (FP32 accumulators).
-template <class L, bool SHIFTED, int CHECK, class In>
+// Statistics of one collided node (FP32 accumulators).  WIDE: the kinetic
+// energy of the FP32 moments in double-float, as exact as in FP64 and off
+// the FP64 pipe, whose ~25 instructions of 64 cycles per node with sums and
+// a division made up an eighth of a 32^3 step.
+template <class L, bool SHIFTED, int CHECK, bool WIDE, class In, class A>
 __device__ __forceinline__ void diag32(const N32<L>& r, In in, double rho0,
-                                       Acc32& acc) {
+                                       A& acc) {
   acc.nodes += 1;
   acc.drho.add(r.drho);
   acc.j0.add(r.j[0]);
   acc.j1.add(r.j[1]);
   acc.j2.add(r.j[2]);
-  acc.ke.add(0.5f * (r.j[0] * r.j[0] + r.j[1] * r.j[1] + r.j[2] * r.j[2]) /
-             r.rho);
+  if constexpr (WIDE) {
+    DF<float> q = df_add(two_prod(r.j[0], r.j[0]), two_prod(r.j[1], r.j[1]));
+    if (L::D == 3) q = df_add(q, two_prod(r.j[2], r.j[2]));
+    q = df_div(q, DF<float>{r.rho, 0.0f});
+    acc.ke.add(DF<float>{0.5f * q.hi, 0.5f * q.lo});
+  } else {
+    acc.ke.add(0.5f * (r.j[0] * r.j[0] + r.j[1] * r.j[1] + r.j[2] * r.j[2]) /
+               r.rho);
+  }
   acc.asum.add(r.alpha);
   acc.amin = fminf(acc.amin, r.alpha);
   acc.amax = fmaxf(acc.amax, r.alpha);
@@ -267,10 +307,11 @@ __device__ __forceinline__ void diag32(const N32<L>& r, In in, double rho0,
 // second stage completes the node); or kNodeFar (nothing written: the FP64
 // fixup collides it).  With aprov null an undecided node keeps its
 // certified alpha.
-template <class L, bool SHIFTED, int DIAG, int CHECK, class In, class Out>
+template <class L, bool SHIFTED, int DIAG, int CHECK, class In, class A,
+          class Out>
 __device__ __forceinline__ unsigned sc32_node_in(
     In in, float rho0f, double rho0, float beta, float corr_rho,
-    const float* __restrict__ corr, float* amap, Acc32& acc, Out out,
+    const float* __restrict__ corr, float* amap, A& acc, Out out,
     float* aprov = nullptr) {
   constexpr int P = npairs<L>();
   float d0, a_extra;
@@ -291,7 +332,7 @@ __device__ __forceinline__ unsigned sc32_node_in(
     r.flags = (r.flags & NF_DEGENERATE) ? NF_DEGENERATE : NF_FORMULA | NF_BAND;
   }
   if (amap) *amap = r.alpha;
-  if (DIAG) diag32<L, SHIFTED, CHECK>(r, in, rho0, acc);
+  if (DIAG) diag32<L, SHIFTED, CHECK, false>(r, in, rho0, acc);
   return kNodeDone;
 }
 
@@ -372,12 +413,13 @@ __device__ __forceinline__ void defer_nodes(unsigned* count, unsigned* queue,
 }
 
 // Same, with the values in a shared-memory column of stride TB.
-template <class L, bool SHIFTED, int DIAG, int CHECK, int TB, class Out>
+template <class L, bool SHIFTED, int DIAG, int CHECK, int TB, class A,
+          class Out>
 __device__ __forceinline__ unsigned sc32_node(const float* sm, float rho0f,
                                           double rho0, float beta,
                                           float corr_rho,
                                           const float* __restrict__ corr,
-                                          float* amap, Acc32& acc, Out out,
+                                          float* amap, A& acc, Out out,
                                           float* aprov = nullptr) {
   return sc32_node_in<L, SHIFTED, DIAG, CHECK>(
       [&](int i) { return sm[i * TB]; }, rho0f, rho0, beta, corr_rho, corr,
@@ -515,18 +557,18 @@ __device__ __forceinline__ void list_open(const StepParams& p, bool mine,
 // per SM; D3Q27 would spill), and it spares the record, its reading and a
 // launch: in a thin shear layer 76 % of the nodes are undecided at every
 // step.  1024^2 shear layer, 50 steps: 4.43 -> 3.47 ms (GB300).
-template <class L, bool SHIFTED, int DIAG, int CHECK, class In, class Out>
+template <class L, bool SHIFTED, int DIAG, int CHECK, class In, class A,
+          class Out>
 __device__ __forceinline__ unsigned refine_inline(const StepParams& p, In in,
                                                   unsigned node, unsigned st,
-                                                  float ap, Acc32& acc,
-                                                  Out out) {
+                                                  float ap, A& acc, Out out) {
   int stage = kStageDone;
   if (st == kNodeRefine)
     stage = second_stage32<L, SHIFTED, DIAG, CHECK>(
         in, p.rho0f, p.betaf, p.corr_rho, p.corr,
         p.alpha_map ? p.alpha_map + node : nullptr, ap, out,
         [&](const N32<L>& r) {
-          if (DIAG) diag32<L, SHIFTED, CHECK>(r, in, p.rho0, acc);
+          if (DIAG) diag32<L, SHIFTED, CHECK, true>(r, in, p.rho0, acc);
         });
   list_open(p, stage == kStageRetry, node);
   return stage == kStageFP64 ? kNodeFar
@@ -543,7 +585,7 @@ __global__ void __launch_bounds__(kSc32Threads, L::Q == 9 && !CHECK ? 3 : 2)
   const unsigned ntiles = (unsigned)((p.n + kSc32Threads - 1) / kSc32Threads);
   const float rho0f = p.rho0f;
   const float beta = p.betaf;
-  Acc32 acc;
+  AccSc<L> acc;
   if (DIAG) acc.init();
   refine_block_begin(&s_refine);
 

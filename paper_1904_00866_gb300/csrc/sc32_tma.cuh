@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(256, 2) k_sc32_tma(const StepParams p) {
       if (t < ntiles) tma_produce<L>(p, smem + k * Q * kTmaRow, &full[k], t);
     }
   }
-  Acc32 acc;
+  AccSc<L> acc;
   if (DIAG) acc.init();
   bool timed_out = false;
   unsigned k = 0;

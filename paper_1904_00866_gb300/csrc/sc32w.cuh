@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kWideThreads, 3)
   const unsigned nwarps = gridDim.x * kWideWarps;
   const float rho0f = p.rho0f;
   const float beta = p.betaf;
-  Acc32 acc;
+  AccSc<L> acc;
   if (DIAG) acc.init();
   __shared__ unsigned s_refine;     // this block's undecided-node entries
   refine_block_begin(&s_refine);
