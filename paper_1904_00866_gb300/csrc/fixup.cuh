@@ -138,8 +138,9 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
 // by their whole warp (formula64_warp, one population per lane), or one per
 // lane when a warp has more than 16, collected 32 at a time on a queue
 // longer than the grid (the first step after initialisation).  On steps with
-// the FP64 entropy check (CHECK) they run on their own lanes, as the check's
-// statistics need each node's populations in one thread.
+// the FP64 entropy check (CHECK) the logarithms run on their own lanes, so
+// that the check repeats their very sums (a tie would otherwise count as a
+// mismatch by rounding); the series forms are the other steps'.
 //
 // Bound by latency: a short list is one chain per warp, and by the fetch of
 // straight-line code that each warp runs once.  A few open nodes run one
@@ -168,6 +169,19 @@ __device__ __forceinline__ void near64_gather(const StepParams& p, int x, int y,
     f[i] = load64<L, half_t>(reinterpret_cast<const half_t*>(
                                  p.in_pop[i])[src_index<L>(p, i, x, y, z)],
                              i, p.rho0, false);
+}
+
+// FP64 entropy check (Eq. (7)) of a node at the alpha it took, from its stored
+// values in f_in.
+template <class L, class S>
+__device__ __noinline__ Check64 check_stored(const StepParams& p,
+                                             long long node, double alpha) {
+  int x, y, z;
+  node_xyz<L>(p, (unsigned)node, x, y, z);
+  Node64<L> c;
+  near64_gather<L>(p, x, y, z, static_cast<const S*>(nullptr), c.f);
+  node64_prepare(c);
+  return node64_check(c, alpha);
 }
 
 // Entries of a list of `count` that a warp of `warps` takes per round: runs
@@ -252,9 +266,15 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
     if (DIAG) acc.far += 1;
     collide64<L, MODE_FORMULA, CHECK>(nd, p, true, acc, DIAG != 0, store_s);
   };
+  auto check = [&](long long node, double alpha, unsigned flags) {
+    const Check64 ck = check_stored<L, S>(p, node, alpha);
+    acc.add_check(ck.h, ck.violation, decision_mismatch(flags, ck.accept_ref),
+                  fabs(alpha - ck.alpha_ref));
+  };
   // FP64 FORMULA of node nd by the whole warp (every lane calls): the series
-  // form when `near` and it settles the node, else the logarithm form
-  auto fp64_warp = [&](long long nd, bool near) {
+  // form when `near` and it settles the node, else the logarithm form; with
+  // CHECK the series form only.  Returns whether the node is done.
+  auto fp64_warp = [&](long long nd, bool near, Warp64& r) {
     int x, y, z;
     coords(nd, x, y, z);
     double f = 0.0;
@@ -280,9 +300,9 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
       else
         p.out_pop[lane][nd] = (float)(p.unshifted ? val : val - lp.w * p.rho0);
     };
-    Warp64 r;
     const bool settled =
         near && near64_warp<L>(lp, lane, f, p.beta, r, store);
+    if (CHECK && !settled) return false;
     if (!settled) r = formula64_warp<L>(lp, f, p.beta, store);
     if (lane == 0) {
       if (DIAG) acc.far += !settled;
@@ -296,6 +316,7 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
         }
       }
     }
+    return true;
   };
   // FP64 series FORMULA of one node in this thread; false: not settled
   auto near_lane = [&](long long node) {
@@ -324,16 +345,7 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
       const double rho = nd.rho * nd.unit;
       acc.add_moments(rho - p.rho0, j, rho);
       acc.add_alpha(alpha, flags, 0);
-      if (CHECK) {
-        Node64<L> c;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) c.f[i] = nd.f[i];
-        node64_prepare(c);
-        const Check64 ck = node64_check(c, alpha);
-        acc.add_check(ck.h, ck.violation,
-                      decision_mismatch(flags, ck.accept_ref),
-                      fabs(alpha - ck.alpha_ref));
-      }
+      if (CHECK) check(node, alpha, flags);
     }
     return true;
   };
@@ -357,7 +369,7 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
   // one per lane costs less FP64 issue in bulk.
   auto logarithms = [&](bool need64, long long node, bool near) {
     const unsigned m64 = __ballot_sync(0xffffffffu, need64);
-    if (CHECK != 0 || (!bulk && !near && __popc(m64) > 16)) {
+    if (CHECK ? !near : (!bulk && !near && __popc(m64) > 16)) {
       if (need64) fp64_lane(node);
     } else if (bulk && !near) {
       const int nk = __popc(m64);
@@ -367,10 +379,23 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
       npend += nk;
     } else {
       unsigned m = m64;
+      double alpha = 2.0;      // with CHECK: what this lane's node took
+      unsigned flags = 0u;
       while (m) {
         const int src_lane = __ffs(m) - 1;
         m &= m - 1;
-        fp64_warp(__shfl_sync(0xffffffffu, node, src_lane), near);
+        Warp64 r;
+        const bool done =
+            fp64_warp(__shfl_sync(0xffffffffu, node, src_lane), near, r);
+        if (CHECK && done && lane == src_lane) {
+          alpha = r.alpha;
+          flags = r.flags;
+          need64 = false;
+        }
+      }
+      if (CHECK) {
+        if (flags != 0u) check(node, alpha, flags);
+        if (need64) fp64_lane(node);
       }
     }
   };
@@ -444,7 +469,7 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
     }
     // a warp with few such nodes runs them in turn, one population per lane
     const bool few =
-        CHECK == 0 && __popc(__ballot_sync(0xffffffffu, direct)) <= kFewOpen;
+        __popc(__ballot_sync(0xffffffffu, direct)) <= kFewOpen;
     if (!few) direct = direct && !near_lane(sn);
 #pragma unroll 1
     for (int t = 0; t < 2; ++t)
@@ -455,7 +480,8 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
     if (npend > 5) {
       flush();
     } else {
-      for (int j = 0; j < npend; ++j) fp64_warp((long long)pend[j], false);
+      Warp64 r;   // (with CHECK nothing is pending)
+      for (int j = 0; j < npend; ++j) fp64_warp((long long)pend[j], false, r);
     }
   }
   if (DIAG) acc.block_reduce_store(p.partials);

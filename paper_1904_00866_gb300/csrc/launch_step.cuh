@@ -63,10 +63,10 @@ static int occupancy_grid(Kernel k, int block, int smem, long long blocks,
   return g < 1 ? 1 : (int)g;
 }
 
-template <class L, class T, int MODE, int DIAG, int CHECK>
+template <class L, int MODE, int DIAG, int CHECK>
 static cudaError_t launch_one(const StepParams& p, int grid, int block,
                               cudaStream_t s, int* grid_used) {
-  auto k = k_stream_collide<L, T, MODE, DIAG, CHECK>;
+  auto k = k_stream_collide<L, MODE, DIAG, CHECK>;
   static ResidentBlocks resident;
   if (grid <= 0)
     grid = occupancy_grid(k, block, 0, (p.tiles * 32 + block - 1) / block,
@@ -81,10 +81,10 @@ static cudaError_t launch_one(const StepParams& p, int grid, int block,
 // blocks per SM), or one warp per block while that spreads the nodes over
 // more SMs: the FP64 pipes then see one warp each instead of four blocks'
 // worth on a few SMs.
-template <class L, class T, int MODE, int DIAG>
+template <class L, class T, int MODE, int DIAG, int CHECK>
 static cudaError_t launch_sc64(const StepParams& p, cudaStream_t s,
                                int* grid_used) {
-  auto k = k_sc64<L, T, MODE, DIAG>;
+  auto k = k_sc64<L, T, MODE, DIAG, CHECK>;
   static ResidentBlocks resident;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -103,13 +103,14 @@ template <class L, class T, int MODE>
 static cudaError_t launch_diag(int diag, int check, const StepParams& p,
                                int grid, int block, cudaStream_t s,
                                int* grid_used) {
-  if (check) return launch_one<L, T, MODE, 1, 1>(p, grid, block, s, grid_used);
   if constexpr (L::D == 1) {
-    if (diag) return launch_one<L, T, MODE, 1, 0>(p, grid, block, s, grid_used);
-    return launch_one<L, T, MODE, 0, 0>(p, grid, block, s, grid_used);
+    if (check) return launch_one<L, MODE, 1, 1>(p, grid, block, s, grid_used);
+    if (diag) return launch_one<L, MODE, 1, 0>(p, grid, block, s, grid_used);
+    return launch_one<L, MODE, 0, 0>(p, grid, block, s, grid_used);
   } else {
-    if (diag) return launch_sc64<L, T, MODE, 1>(p, s, grid_used);
-    return launch_sc64<L, T, MODE, 0>(p, s, grid_used);
+    if (check) return launch_sc64<L, T, MODE, 1, 1>(p, s, grid_used);
+    if (diag) return launch_sc64<L, T, MODE, 1, 0>(p, s, grid_used);
+    return launch_sc64<L, T, MODE, 0, 0>(p, s, grid_used);
   }
 }
 
@@ -272,9 +273,8 @@ static cudaError_t launch_sc16(int diag, int check, const StepParams& p,
   return launch_sc16_one<L, 0, 0>(p, grid, s, grid_used);
 }
 
-// The fixup grid must equal the grid of the FP32 / FP16 step when DIAG is
-// set (its partials rows follow the step's rows); without DIAG any grid
-// works.  S: storage type (float or half_t).
+// Any grid works; with DIAG each block writes one row of partials.  S:
+// storage type (float or half_t).
 template <class L, class S = float>
 static cudaError_t launch_far_lattice(int diag, int check,
                                       const StepParams& p, int grid,

@@ -20,6 +20,7 @@
 // before or nearer (1.3e-15 against 1.4e-15 on 128^3).
 #pragma once
 #include "fp16_storage.cuh"
+#include "sc32.cuh"
 #include "series64.cuh"
 #include "stats.cuh"
 #include "stream_collide.cuh"
@@ -33,15 +34,35 @@ struct Collided64 {
   int iters;
 };
 
-template <class L>
-__device__ __forceinline__ void pull_sources(const StepParams& p,
-                                             unsigned node, int& x, int& y,
-                                             int& z) {
-  const unsigned q1 = p.div_nx.div(node);
-  x = (int)(node - q1 * (unsigned)p.nx);
-  const unsigned q2 = p.div_ny.div(q1);
-  y = (int)(q1 - q2 * (unsigned)p.ny);
-  z = (int)q2;
+// The populations of a node from its stored values in f_in.
+template <class L, class T>
+__device__ __forceinline__ void gather64(const StepParams& p, unsigned node,
+                                         double (&f)[L::Q]) {
+  const T* fin = static_cast<const T*>(p.f_in);
+  int x, y, z;
+  node_xyz<L>(p, node, x, y, z);
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const T v = fin[(long long)i * p.ps + src_index<L>(p, i, x, y, z)];
+    if constexpr (sizeof(T) == 8)
+      f[i] = v;
+    else if constexpr (sizeof(T) == 2)
+      f[i] = h16_to_f<L>(v, i, p.rho0);
+    else
+      f[i] = p.unshifted ? (double)v : L::w(i) * p.rho0 + (double)v;
+  }
+}
+
+// FP64 entropy check (Eq. (7)) of a node at the alpha it took, by either
+// path; out of line, so that a checked step differs from the others in its
+// statistics only.
+template <class L, class T>
+__device__ __noinline__ Check64 check64_at(const StepParams& p, unsigned node,
+                                           double alpha) {
+  Node64<L> nd;
+  gather64<L, T>(p, node, nd.f);
+  node64_prepare(nd);
+  return node64_check(nd, alpha);
 }
 
 // The logarithm path of one node, from its stored values in f_in.  Flags
@@ -49,21 +70,9 @@ __device__ __forceinline__ void pull_sources(const StepParams& p,
 template <class L, class T, int MODE>
 __device__ __noinline__ Collided64 far64_node(const StepParams& p,
                                               unsigned node) {
-  const T* fin = static_cast<const T*>(p.f_in);
   T* fout = static_cast<T*>(p.f_out);
-  int x, y, z;
-  pull_sources<L>(p, node, x, y, z);
   Node64<L> nd;
-#pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
-    const T v = fin[(long long)i * p.ps + src_index<L>(p, i, x, y, z)];
-    if constexpr (sizeof(T) == 8)
-      nd.f[i] = v;
-    else if constexpr (sizeof(T) == 2)
-      nd.f[i] = h16_to_f<L>(v, i, p.rho0);
-    else
-      nd.f[i] = p.unshifted ? (double)v : L::w(i) * p.rho0 + (double)v;
-  }
+  gather64<L, T>(p, node, nd.f);
   Collided64 r;
   r.iters = 0;
   r.alpha = 2.0;
@@ -96,7 +105,7 @@ __device__ __noinline__ Collided64 far64_node(const StepParams& p,
   return r;
 }
 
-template <class L, class T, int MODE, int DIAG>
+template <class L, class T, int MODE, int DIAG, int CHECK>
 __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
   chain_begin();
   constexpr int Q = L::Q;
@@ -104,13 +113,18 @@ __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
   T* fout = static_cast<T*>(p.f_out);
   Acc acc;
   if (DIAG) acc.init();
+  auto check = [&](unsigned node, double alpha, unsigned flags) {
+    const Check64 ck = check64_at<L, T>(p, node, alpha);
+    acc.add_check(ck.h, ck.violation, decision_mismatch(flags, ck.accept_ref),
+                  fabs(alpha - ck.alpha_ref));
+  };
   for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < p.n;
        k += (long long)gridDim.x * blockDim.x) {
     const unsigned node = (unsigned)k;
     Near64<L> nd;
     {
       int x, y, z;
-      pull_sources<L>(p, node, x, y, z);
+      node_xyz<L>(p, node, x, y, z);
       // element offsets of the neighbours along each axis
       const int dx[3] = {x == p.nx - 1 ? 1 - p.nx : 1, 0,
                          x == 0 ? p.nx - 1 : -1};
@@ -162,6 +176,7 @@ __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
                            nd.j[2] * nd.j[2]);
         acc.add_moments_ke(fma(nd.rho, nd.unit, -p.rho0), j, 0.5 * ke);
         acc.add_alpha(alpha, flags, iters);
+        if (CHECK) check(node, alpha, flags);
       }
     } else {
       const Collided64 c = far64_node<L, T, MODE>(p, node);
@@ -170,6 +185,7 @@ __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
         if (DIAG) {
           acc.add_moments(c.rho - p.rho0, c.j, c.rho);
           acc.add_alpha(c.alpha, c.flags, c.iters);
+          if (CHECK) check(node, c.alpha, c.flags);
         }
       }
     }

@@ -1,5 +1,6 @@
 // Fused pull-scheme stream + collide kernel (Eq. (5b) gather, Eq. (5a)
-// relax) for one periodic lattice.
+// relax) for one periodic lattice of FP64 populations, and the parameters all
+// stream-collide kernels take.
 //
 // Storage: SoA populations [Q][nz][ny][nx], x fastest.  The buffer holds the
 // post-collision values f~ of the previous step; the pre-collision state at
@@ -8,12 +9,10 @@
 //
 // Work decomposition: a tile is 32 consecutive x-nodes of one (y, z) row,
 // one warp per tile; warps stride over tiles (grid sized to the SM count).
-// The 27 (or 9) gathers of a tile are warp-coalesced 128-byte rows; the
-// +-1 x-shift of a row is absorbed by L1/L2.
+// The gathers of a tile are warp-coalesced rows; the +-1 x-shift of a row is
+// absorbed by L1/L2.
 //
-// Template parameters: lattice L, storage type T (double: FP64 arithmetic
-// for every alpha mode; float / half_t: FP32 or FP16-shifted storage with
-// ROOT / SECANT in FP64 -- their FORMULA runs in the pipelined k_sc32 /
+// Template parameters: lattice L (D1Q3; the others run in k_sc64, k_sc32 and
 // k_sc16), alpha MODE, DIAG (fused statistics), CHECK (FP64 entropy check;
 // implies DIAG).
 #pragma once
@@ -160,15 +159,15 @@ __device__ __forceinline__ void collide64(Node64<L>& nd, const StepParams& p,
   if (p.alpha_map) store(-1, alpha);
 }
 
-template <class L, class T, int MODE, int DIAG, int CHECK>
+template <class L, int MODE, int DIAG, int CHECK>
 __global__ void __launch_bounds__(256)
     k_stream_collide(const StepParams p) {
   constexpr int Q = L::Q;
   const int lane = threadIdx.x & 31;
   const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  const T* __restrict__ fin = static_cast<const T*>(p.f_in);
-  T* __restrict__ fout = static_cast<T*>(p.f_out);
+  const double* __restrict__ fin = static_cast<const double*>(p.f_in);
+  double* __restrict__ fout = static_cast<double*>(p.f_out);
   Acc acc;
   acc.init();
 
@@ -177,53 +176,17 @@ __global__ void __launch_bounds__(256)
     tile_coords<L>(p, t, lane, x, y, z);
     if (x >= p.nx) continue;
     const long long node = ((long long)z * p.ny + y) * p.nx + x;
-
-    T v[Q];
+    Node64<L> nd;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) v[i] = fin[(long long)i * p.ps + src_index<L>(p, i, x, y, z)];
-
-    auto store_T = [&](int i, double val) {
-      if (i < 0) {
-        p.alpha_map[node] = (float)val;
-      } else {
-        fout[(long long)i * p.ps + node] = (T)val;
-      }
-    };
-
-    if constexpr (sizeof(T) == 8) {
-      // ---------------- FP64 storage: FP64 arithmetic -------------------
-      Node64<L> nd;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) nd.f[i] = (double)v[i];
-      collide64<L, MODE, CHECK>(nd, p, false, acc, DIAG != 0, store_T);
-    } else if constexpr (MODE != MODE_FORMULA) {
-      // ------------- FP32 storage, ROOT / SECANT in FP64 -----------------
-      Node64<L> nd;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const double s = L::w(i) * p.rho0;
-        if constexpr (sizeof(T) == 2)
-          nd.f[i] = h16_to_f<L>(v[i], i, p.rho0);
-        else
-          nd.f[i] = p.unshifted ? (double)v[i] : s + (double)v[i];
-      }
-      auto store_s = [&](int i, double val) {
-        if (i < 0) {
-          p.alpha_map[node] = (float)val;
-        } else {
-          const double s = L::w(i) * p.rho0;
-          if constexpr (sizeof(T) == 2)
-            fout[(long long)i * p.ps + node] = h16_from_dev<L>(val - s, i);
-          else
-            fout[(long long)i * p.ps + node] =
-                (T)(p.unshifted ? val : val - s);
-        }
-      };
-      collide64<L, MODE, CHECK>(nd, p, true, acc, DIAG != 0, store_s);
-    } else {
-      static_assert(sizeof(T) == 8 || MODE != MODE_FORMULA,
-                    "FP32 / FP16 FORMULA runs in k_sc32 / k_sc16");
-    }
+    for (int i = 0; i < Q; ++i)
+      nd.f[i] = fin[(long long)i * p.ps + src_index<L>(p, i, x, y, z)];
+    collide64<L, MODE, CHECK>(nd, p, false, acc, DIAG != 0,
+                              [&](int i, double val) {
+                                if (i < 0)
+                                  p.alpha_map[node] = (float)val;
+                                else
+                                  fout[(long long)i * p.ps + node] = val;
+                              });
   }
   if (DIAG) acc.block_reduce_store(p.partials);
 }
