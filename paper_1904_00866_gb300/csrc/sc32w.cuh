@@ -126,14 +126,21 @@ __global__ void __launch_bounds__(kWideThreads, 3)
       const int t = 32 * h + lane;
       const unsigned node = seg * kWideSeg + t;
       auto in = [&](int i) { return st[wide_base<L>(i) + wide_shift<L>(i) + t]; };
+      auto out = [&](int i, float v) { p.out_pop[i][node] = v; };
       float ap = 0.0f;
-      const unsigned res = sc32_node_in<L, true, DIAG, CHECK>(
+      unsigned res = sc32_node_in<L, true, DIAG, CHECK>(
           in, rho0f, p.rho0, beta, 0.0f, nullptr,
-          p.alpha_map ? p.alpha_map + node : nullptr, acc,
-          [&](int i, float v) { p.out_pop[i][node] = v; },
+          p.alpha_map ? p.alpha_map + node : nullptr, acc, out,
           p.exact ? &ap : nullptr);
-      if (p.exact)
-        defer_undecided<L>(p, &s_refine, res == kNodeRefine, in, node, ap);
+      // D2Q9: the second stage here, as in k_sc32 (no record buffer)
+      if constexpr (L::Q == 9) {
+        if (p.exact)
+          res = refine_inline<L, true, DIAG, CHECK>(p, in, node, res, ap, acc,
+                                                    out);
+      } else {
+        if (p.exact)
+          defer_undecided<L>(p, &s_refine, res == kNodeRefine, in, node, ap);
+      }
       defer_nodes(&p.far_count[p.parity], p.far_queue, p.far_cap,
                   p.err_flags, node, res == kNodeFar ? kNodeFar : kNodeDone);
     }
