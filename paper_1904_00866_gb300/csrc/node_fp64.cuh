@@ -111,7 +111,7 @@ __device__ __forceinline__ unsigned node64_prepare(Node64<L>& s) {
   if (L::D < 2) s.j[1] = 0.0;
   if (!(rho > 0.0) || !isfinite(rho)) bad |= NF_BAD_NONFINITE;
   s.rho = rho;
-  double amax = INFINITY;
+  double xmin = 0.0;
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
     double P = rho * L::w(i);
@@ -122,9 +122,11 @@ __device__ __forceinline__ unsigned node64_prepare(Node64<L>& s) {
     }
     const double x = (P - s.f[i]) / s.f[i];
     s.x[i] = x;
-    if (x < 0.0) amax = fmin(amax, -1.0 / x);
+    xmin = fmin(xmin, x);
   }
-  s.amax = amax;
+  // min over x_i < 0 of -1 / x_i: rounding is monotone, so the smallest x_i
+  // gives the smallest quotient, and one division does
+  s.amax = xmin < 0.0 ? -1.0 / xmin : INFINITY;
   return bad;
 }
 

@@ -5,9 +5,11 @@
 // nodes of the flat index (ragged rows leave no lane idle).  Nodes near
 // equilibrium take the series path (series64.cuh: ~120 FP64 instructions
 // per D3Q27 FORMULA node and 60 per D2Q9 node, at 64 cycles each the
-// kernel's bound: FP64 pipe 84 % busy for D2Q9), the others re-gather
-// their populations and take the logarithm path (node_fp64.cuh) out of
-// line, so that its registers do not count here.
+// kernel's bound: FP64 pipe 84 % busy for D2Q9, about 60 % for D3Q27, whose
+// FP32 and integer part does not overlap with it at two warps per scheduler).
+// The others take the logarithm path (node_fp64.cuh) out of line, so that its
+// registers do not count here: each warp collects them in shared memory and
+// runs them 32 at a time, one per lane, from their stored values.
 //
 // Measured (GB300, us per step; before: every node through the logarithm
 // path, one row segment of 32 nodes per warp, ~700 FP64 instructions per
@@ -15,7 +17,15 @@
 //   D2Q9 1024^2 shear layer, FP64 storage, FORMULA     1326 ->  128
 //   D2Q9 1024^2 shear layer, FP32 storage, ROOT       11560 ->  565
 //   D3Q27 128^3 Taylor-Green, FP64 storage, FORMULA    7960 ->  667
-//   D2Q9 64^2, FP64 storage, FORMULA with statistics     69 ->   12
+//   D2Q9 64^2, FP64 storage, FORMULA with statistics     69 ->   10
+// One FORMULA step with a share of the nodes at |x| ~ 0.2, all through the
+// logarithm path -> each warp's far nodes where it meets them -> collected:
+//   D3Q27 96^3    1 %  6449 -> 3574 ->  509     D2Q9 1024^2  1504 ->  752 ->  274
+//                10 %  7026 -> 9142 -> 1437                  1824 -> 1842 ->  447
+//               100 %  5481 -> 6291 -> 5975                  2039 -> 2169 -> 2084
+// (a state with every node far pays for the attempt, and with ROOT for the 12
+// warps per SM: D2Q9 43.7 -> 46.8 ms; the first step after initialisation,
+// all by logarithms, takes what it took).
 // Populations after 8 to 54 steps are as far from the 64-bit reference as
 // before or nearer (1.3e-15 against 1.4e-15 on 128^3).
 #pragma once
@@ -118,11 +128,20 @@ __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
     acc.add_check(ck.h, ck.violation, decision_mismatch(flags, ck.accept_ref),
                   fabs(alpha - ck.alpha_ref));
   };
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < p.n;
-       k += (long long)gridDim.x * blockDim.x) {
+  // this warp's nodes for the logarithm path (warp-uniform count, below 32
+  // before a round adds up to 32)
+  __shared__ unsigned far_s[4][64];   // blocks of up to 128 threads
+  unsigned* far = far_s[threadIdx.x >> 5];
+  int nfar = 0;
+  const int lane = threadIdx.x & 31;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long k0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+       k0 < p.n || nfar > 0; k0 += stride) {
+    const long long k = k0 + lane;
     const unsigned node = (unsigned)k;
+    bool is_far = k < p.n;
     Near64<L> nd;
-    {
+    if (k < p.n) {
       int x, y, z;
       node_xyz<L>(p, node, x, y, z);
       // element offsets of the neighbours along each axis
@@ -142,8 +161,9 @@ __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
       }
     }
     Series64 se;
-    if (near64_prepare(
-            nd, se, sizeof(T) == 8 ? kSeriesXMax : kSeriesXMaxRounded)) {
+    if (is_far && near64_prepare(nd, se, sizeof(T) == 8 ? kSeriesXMax
+                                                        : kSeriesXMaxRounded)) {
+      is_far = false;
       unsigned flags = 0;
       int iters = 0;
       double alpha = 2.0;
@@ -178,14 +198,26 @@ __global__ void __launch_bounds__(128) k_sc64(const StepParams p) {
         acc.add_alpha(alpha, flags, iters);
         if (CHECK) check(node, alpha, flags);
       }
-    } else {
-      const Collided64 c = far64_node<L, T, MODE>(p, node);
-      if (!(c.flags & (NF_BAD_NEG | NF_BAD_NONFINITE))) {
-        if (p.alpha_map) p.alpha_map[k] = (float)c.alpha;
-        if (DIAG) {
-          acc.add_moments(c.rho - p.rho0, c.j, c.rho);
-          acc.add_alpha(c.alpha, c.flags, c.iters);
-          if (CHECK) check(node, c.alpha, c.flags);
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, is_far);
+    if (is_far) far[nfar + __popc(m & ((1u << lane) - 1u))] = node;
+    nfar += __popc(m);
+    if (nfar >= 32 || (nfar > 0 && k0 + stride >= p.n)) {   // warp-uniform
+      const int take = min(nfar, 32);
+      nfar -= take;
+      __syncwarp();
+      const bool mine = lane < take;
+      const unsigned fn = mine ? far[nfar + lane] : 0u;
+      __syncwarp();
+      if (mine) {
+        const Collided64 c = far64_node<L, T, MODE>(p, fn);
+        if (!(c.flags & (NF_BAD_NEG | NF_BAD_NONFINITE))) {
+          if (p.alpha_map) p.alpha_map[fn] = (float)c.alpha;
+          if (DIAG) {
+            acc.add_moments(c.rho - p.rho0, c.j, c.rho);
+            acc.add_alpha(c.alpha, c.flags, c.iters);
+            if (CHECK) check(fn, c.alpha, c.flags);
+          }
         }
       }
     }
