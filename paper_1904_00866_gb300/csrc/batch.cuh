@@ -587,14 +587,17 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
       }
     }
   };
-  // rounds as in k_far_fixup
-  const unsigned use = open_warps(open_count, gridDim.x);
+  // rounds as in k_far_fixup (a list of both lattices: D3Q27's limit)
+  constexpr unsigned kFew = few_open<D3Q27>();
+  const unsigned use = open_warps(open_count, gridDim.x, kFew);
+  const bool few_o = few_listed(open_count, gridDim.x, kFew);
+  const bool few_q = few_queued(count, W);
   const unsigned WO = gridDim.x * use;
   const unsigned run_o = run_length(open_count, WO);
   const unsigned run_q = run_length(count, W);
   unsigned base_o = (unsigned)warp < use ? 0u : open_count, base_q = 0u;
   for (;;) {
-    bool need64 = false, open = false, direct = false;
+    bool need64 = false, open = false, direct = false, few = few_o;
     unsigned long long e = 0;
     if (base_o < open_count) {
       const unsigned k = base_o +
@@ -655,13 +658,12 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
     if (nnear >= 32 || (nnear > 0 && base_q >= count)) {
       const int take = min(nnear, 32);
       nnear -= take;
+      few = few_q;
       __syncwarp();
       direct = lane < take;
       if (direct) sn = near[nnear + lane];
       __syncwarp();
     }
-    const bool few =
-        __popc(__ballot_sync(0xffffffffu, direct)) <= kFewOpen;
     if (!few) direct = direct && !near_lane(sn);
 #pragma unroll 1
     for (int t = 0; t < 2; ++t)

@@ -145,7 +145,10 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
 // Bound by latency: a short list is one chain per warp, and by the fetch of
 // straight-line code that each warp runs once.  A few open nodes run one
 // at a time (near64_warp), many one per lane (near64_formula: up to 32 nodes
-// for ~120 FP64 instructions of 64 cycles).  Before, the second stage ran
+// for ~120 FP64 instructions of 64 cycles); the form is the list's, so the
+// same input gives the same alphas.  (Logarithm nodes of a queue of more than
+// 16 per warp and round take the form their warp's share asks for: their sums,
+// and a tie's branch, may then differ by rounding between runs.)  Before, the second stage ran
 // again with double-float leading terms (~3,000 FP32 instructions) and what
 // that left took the logarithms, ~460 FP64 instructions a node.  Entries are
 // dealt evenly as runs of neighbours; the grid is one block per SM (the
@@ -190,16 +193,36 @@ __device__ __forceinline__ unsigned run_length(unsigned count, unsigned warps) {
   return min(32u, (count + warps - 1u) / warps);
 }
 
-// Open nodes a warp settles one at a time (near64_warp, ~2.5 us each) rather
-// than one per lane (~25 us for D3Q27, ~10 us for D2Q9, however few).
-constexpr int kFewOpen = 8;
+// Open nodes per warp up to which they run one at a time (near64_warp) rather
+// than one per lane (near64_formula).  us per step of 64,250 (D2Q9) and
+// 65,600 (D3Q27) nodes with 1, 2, 5, 6 and 16 open nodes per warp, GB300:
+//   D2Q9   in turn 27.1 34.4 57.3 63.9 136   per lane 28.1 28.9 30.1 29.3 29.9
+//   D3Q27  in turn 36.3 41.7 57.4 66.7 114   per lane 51.8 55.1 58.3 61.0 71.1
+template <class L>
+__host__ __device__ constexpr unsigned few_open() {
+  return L::Q == 9 ? 1u : 5u;
+}
+// The form is the whole list's, not a warp's: which entries share a warp is
+// the order of atomic additions, and alphas of the two forms (~1e-15 apart)
+// may round down to different FP32 numbers, so a choice per warp would let two
+// runs of one input differ.
+__device__ __forceinline__ bool few_listed(unsigned count, unsigned blocks,
+                                           unsigned few) {
+  return count <= blocks * (8u * few);
+}
+// Of `count` queued entries, which take the second stage here first, a few
+// per cent are left open in a developed flow (under 2 per warp of two rounds);
+// on a longer queue (the first step after initialisation) lanes fill up.
+__device__ __forceinline__ bool few_queued(unsigned count, unsigned warps) {
+  return count <= 64u * warps;
+}
 // Warps per block that take open nodes: all while each gets few, then one
 // per sub-partition as long as their lanes hold the list (two would share
 // the FP64 pipe for nothing), then all.
-__device__ __forceinline__ unsigned open_warps(unsigned count,
-                                               unsigned blocks) {
-  return count > blocks * (8u * kFewOpen) && count <= blocks * (4u * 32u) ? 4u
-                                                                          : 8u;
+__device__ __forceinline__ unsigned open_warps(unsigned count, unsigned blocks,
+                                               unsigned few) {
+  return !few_listed(count, blocks, few) && count <= blocks * (4u * 32u) ? 4u
+                                                                         : 8u;
 }
 
 template <class L, class S, int DIAG, int CHECK>
@@ -402,13 +425,15 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
   // Rounds over the open-node list, then over the queue, then until the
   // nodes its second stage left are settled; one call site each for the
   // series and the logarithms.
-  const unsigned use = open_warps(open_count, gridDim.x);
+  const unsigned use = open_warps(open_count, gridDim.x, few_open<L>());
+  const bool few_o = few_listed(open_count, gridDim.x, few_open<L>());
+  const bool few_q = few_queued(count, W);
   const unsigned WO = gridDim.x * use;
   const unsigned run_o = run_length(open_count, WO);
   const unsigned run_q = run_length(count, W);
   unsigned base_o = (unsigned)warp < use ? 0u : open_count, base_q = 0u;
   for (;;) {
-    bool need64 = false, open = false, direct = false;
+    bool need64 = false, open = false, direct = false, few = few_o;
     long long node = 0;
     if (base_o < open_count) {
       const unsigned k = base_o +
@@ -462,14 +487,12 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
     if (nnear >= 32 || (nnear > 0 && base_q >= count)) {   // warp-uniform
       const int take = min(nnear, 32);
       nnear -= take;
+      few = few_q;
       __syncwarp();
       direct = lane < take;
       if (direct) sn = (long long)near[nnear + lane];
       __syncwarp();
     }
-    // a warp with few such nodes runs them in turn, one population per lane
-    const bool few =
-        __popc(__ballot_sync(0xffffffffu, direct)) <= kFewOpen;
     if (!few) direct = direct && !near_lane(sn);
 #pragma unroll 1
     for (int t = 0; t < 2; ++t)
