@@ -173,6 +173,22 @@ struct Near64 {
   double unit;
 };
 
+// 3u and s = sqrt(1 + 3u^2) - 1 of one axis; false: |u| >= kUMax32.  One
+// Newton step on s^2 + 2s - 3u^2 = 0 from the FP32 value, whose relative error
+// (< 2^-20) the step squares; the reciprocal of its slope is refined once.
+__device__ __forceinline__ bool axis_near(double u, double& u3, double& sv) {
+  u3 = 3.0 * u;
+  const float uf = d2f_trunc(u);
+  const float yf = fmaf(3.0f * uf, uf, 1.0f);
+  const float s0f = 3.0f * uf * uf * rcp_approx(1.0f + yf * rsqrt_approx(yf));
+  const double s0 = f2d(s0f);
+  const double rs = f2d(rcp_approx(fmaf(2.0f, s0f, 2.0f)));
+  const double g = fma(s0, s0 + 2.0, -u3 * u);
+  const double ri = fma(rs, fma(-fma(2.0, s0, 2.0), rs, 1.0), rs);
+  sv = fma(-g, ri, s0);
+  return fabsf(uf) < kUMax32;
+}
+
 // Moments, n_i and the scaled x moments of a node whose f[] is filled.
 // False: the node is outside the series' range, max |x_i| <= xmax.
 template <class L>
@@ -191,8 +207,10 @@ __device__ __forceinline__ bool near64_prepare(Near64<L>& s, Series64& r,
   if (fmin < (200 << 20) || fmax > (1800 << 20)) return false;
   const int rexp = (fmax & 0x7ff00000) + (3 << 20);
   if (fmin < rexp - (15 << 20)) return false;
-  // Mass and momentum in 64-bit integers: exact, and off the FP64 pipe (49
-  // additions for D3Q27).  Within the series' range f_0 >= 0.2 rho, so rho
+  // Mass and momentum in 64-bit integers: exact but for the bits of a
+  // population below 2^-59 of the largest one's power of two (27 of them stay
+  // below half an ulp of the mass), and off the FP64 pipe (49 additions for
+  // D3Q27).  Within the series' range f_0 >= 0.2 rho, so rho
   // stays below 2^4 of the largest f_i's power of two; a node for which it
   // does not overflows, and its f^eq then differs from f far beyond xmax.
   const int top = rexp + (1 << 20) + 0xfffff;
@@ -231,19 +249,8 @@ __device__ __forceinline__ bool near64_prepare(Near64<L>& s, Series64& r,
   bool slow = false;
 #pragma unroll
   for (int a = 0; a < L::D; ++a) {
-    const double u = s.j[a] * s.inv_rho, u3 = 3.0 * u;
-    const float uf = d2f_trunc(u);
-    slow = slow || !(fabsf(uf) < kUMax32);
-    // s = sqrt(1 + 3u^2) - 1: one Newton step on s^2 + 2s - 3u^2 = 0 from
-    // the FP32 value, whose relative error (< 2^-20) the step squares; the
-    // reciprocal of its slope is refined once
-    const float yf = fmaf(3.0f * uf, uf, 1.0f);
-    const float s0f = 3.0f * uf * uf * rcp_approx(1.0f + yf * rsqrt_approx(yf));
-    const double s0 = f2d(s0f);
-    const double rs = f2d(rcp_approx(fmaf(2.0f, s0f, 2.0f)));
-    const double g = fma(s0, s0 + 2.0, -u3 * u);
-    const double ri = fma(rs, fma(-fma(2.0, s0, 2.0), rs, 1.0), rs);
-    const double sv = fma(-g, ri, s0);
+    double u3, sv;
+    slow = !axis_near(s.j[a] * s.inv_rho, u3, sv) || slow;
     const double b = fma(2.0, sv, 1.0);
     psi[a][2] = b + u3;
     psi[a][0] = b - u3;

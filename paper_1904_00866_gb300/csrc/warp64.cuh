@@ -176,19 +176,7 @@ __device__ __forceinline__ bool near64_warp(const LanePop& lp, int lane,
   const double j = from_fixed(ax == 0 ? jx : (ax == 1 ? jy : jz));
   const double inv_rho = rcp64(rho);
   double u3, sv;
-  {   // as near64_prepare
-    const double u = j * inv_rho;
-    u3 = 3.0 * u;
-    const float uf = d2f_trunc(u);
-    if (__any_sync(kAll, !(fabsf(uf) < kUMax32))) return false;
-    const float yf = fmaf(3.0f * uf, uf, 1.0f);
-    const float s0f = 3.0f * uf * uf * rcp_approx(1.0f + yf * rsqrt_approx(yf));
-    const double s0 = f2d(s0f);
-    const double rs = f2d(rcp_approx(fmaf(2.0f, s0f, 2.0f)));
-    const double g = fma(s0, s0 + 2.0, -u3 * u);
-    const double ri = fma(rs, fma(-fma(2.0, s0, 2.0), rs, 1.0), rs);
-    sv = fma(-g, ri, s0);
-  }
+  if (__any_sync(kAll, !axis_near(j * inv_rho, u3, sv))) return false;
   constexpr double k6i = 1.0 / pow6(L::D);
   double P = rho * __hiloint2double(
                        __double2hiint(k6i) + rexp - ((62 + 1023) << 20),
