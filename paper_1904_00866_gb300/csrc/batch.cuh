@@ -405,7 +405,6 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
   if (count + open_count == 0u) return;
   const int lane = threadIdx.x & 31;
   const unsigned W = gridDim.x * (blockDim.x >> 5);
-  const unsigned wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const LanePop lp27 = lane_pop<D3Q27>(lane), lp9 = lane_pop<D2Q9>(lane);
   const bool bulk = count > gridDim.x * blockDim.x;
   auto coords = [](const MemberDesc& m, unsigned node, int& x, int& y,
@@ -558,24 +557,24 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
     };
     return m.lattice == 1 ? run(D3Q27{}) : run(D2Q9{});
   };
-  __shared__ unsigned long long pend_s[8][32], near_s[8][64];
+  __shared__ unsigned long long pend_s[8][64], near_s[8][64];
   const int warp = threadIdx.x >> 5;
   unsigned long long* pend = pend_s[warp];
   unsigned long long* near = near_s[warp];
   int npend = 0, nnear = 0;
-  auto flush = [&]() {   // every lane calls
+  auto flush = [&]() {   // 32 of them; every lane calls
+    npend -= 32;
     __syncwarp();
-    if (lane < npend) fp64_lane(pend[lane]);
+    fp64_lane(pend[npend + lane]);
     __syncwarp();
-    npend = 0;
   };
   auto logarithms = [&](bool need64, unsigned long long e, bool near) {
     const unsigned m64 = __ballot_sync(0xffffffffu, need64);
-    if (!bulk && !near && __popc(m64) > 16) {
+    if (!bulk && !near && __popc(m64) > 5) {
       if (need64) fp64_lane(e);
     } else if (bulk && !near) {
       const int nk = __popc(m64);
-      if (npend + nk > 32) flush();
+      if (npend + nk > 64) flush();
       if (need64) pend[npend + __popc(m64 & ((1u << lane) - 1u))] = e;
       npend += nk;
     } else {
@@ -600,14 +599,14 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
     bool need64 = false, open = false, direct = false, few = few_o;
     unsigned long long e = 0;
     if (base_o < open_count) {
-      const unsigned k = base_o +
-                         (blockIdx.x * use + (unsigned)warp) * run_o +
-                         (unsigned)lane;
+      const unsigned k =
+          base_o + dealt(bulk, (unsigned)warp) * run_o + (unsigned)lane;
       base_o += run_o * WO;
       direct = (unsigned)lane < run_o && k < open_count;
       if (direct) e = bp.far_queue[bp.far_cap - 1u - k];
     } else if (base_q < count) {
-      const unsigned k = base_q + wid * run_q + (unsigned)lane;
+      const unsigned k =
+          base_q + dealt(bulk, (unsigned)warp) * run_q + (unsigned)lane;
       base_q += run_q * W;
       if ((unsigned)lane < run_q && k < count) {
         e = bp.far_queue[k];
@@ -669,12 +668,31 @@ __global__ void __launch_bounds__(256) k_batch_fixup(const BatchParams bp) {
     for (int t = 0; t < 2; ++t)
       logarithms(t == 0 ? direct : need64, t == 0 ? sn : e, t == 0 && few);
   }
-  if (npend > 0) {   // bulk remainder: few nodes run one per warp
-    __syncwarp();
-    if (npend > 5) {
-      flush();
-    } else {
-      for (int j = 0; j < npend; ++j) fp64_warp(pend[j], false);
+  // What the warps still hold of a long queue, pooled over the block: full
+  // warps of nodes, one per lane, on different sub-partitions (few nodes: one
+  // per warp).
+  if (bulk) {
+    __shared__ unsigned long long pool[8 * 64];
+    __shared__ int held[8];
+    if (lane == 0) held[warp] = npend;
+    __syncthreads();
+    int at = 0, total = 0;
+    for (int w = 0; w < 8; ++w) {
+      if (w < warp) at += held[w];
+      total += held[w];
+    }
+    for (int k = lane; k < npend; k += 32) pool[at + k] = pend[k];
+    __syncthreads();
+    for (int k = 32 * warp; k < total; k += 32 * 8) {
+      const int m = min(32, total - k);
+      const unsigned long long e = lane < m ? pool[k + lane] : 0u;
+      if (m > 5) {
+        if (lane < m) fp64_lane(e);
+      } else {
+        for (int j = 0; j < m; ++j) {
+          fp64_warp(__shfl_sync(0xffffffffu, e, j), false);
+        }
+      }
     }
   }
 }

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
 // here first, one per thread, and what it leaves is collected per warp for
 // the series.  Nodes that need the logarithms are collided one at a time
 // by their whole warp (formula64_warp, one population per lane), or one per
-// lane when a warp has more than 16, collected 32 at a time on a queue
+// lane when a warp has more than five, collected 32 at a time on a queue
 // longer than the grid (the first step after initialisation).  On steps with
 // the FP64 entropy check (CHECK) the logarithms run on their own lanes, so
 // that the check repeats their very sums (a tie would otherwise count as a
@@ -146,9 +146,9 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
 // straight-line code that each warp runs once.  A few open nodes run one
 // at a time (near64_warp), many one per lane (near64_formula: up to 32 nodes
 // for ~120 FP64 instructions of 64 cycles); the form is the list's, so the
-// same input gives the same alphas.  (Logarithm nodes of a queue of more than
-// 16 per warp and round take the form their warp's share asks for: their sums,
-// and a tie's branch, may then differ by rounding between runs.)  Before, the second stage ran
+// same input gives the same alphas.  (Logarithm nodes take the form their
+// warp's share asks for: their sums, and a tie's branch, may differ by
+// rounding between runs.)  Before, the second stage ran
 // again with double-float leading terms (~3,000 FP32 instructions) and what
 // that left took the logarithms, ~460 FP64 instructions a node.  Entries are
 // dealt evenly as runs of neighbours; the grid is one block per SM (the
@@ -156,6 +156,12 @@ __global__ void __launch_bounds__(256, 2) k_refine_stage(const StepParams p,
 // us per launch, before -> now (GB300): D3Q27 256^3 binary16 41 -> 15,
 // 121 x 64 x 70 static step (no buffer) 36 -> 22, D2Q9 1024^2 shear layer
 // 25 -> 12; all open nodes one per lane: static 64.
+// First step after initialisation (every node undecided, the logarithm nodes
+// together in symmetry planes), before the FP64 series -> with partial flushes
+// per warp -> runs dealt across blocks, remainders pooled, ties sent straight
+// to the logarithms: Taylor-Green 96^3 445 -> 703 -> 380, 256^3
+// 4000 -> 4590 -> 3700; random phases 96^3 184 -> 144 -> 155, 256^3
+// 2340 -> 2020 -> 2100.
 template <class L>
 __device__ __forceinline__ void near64_gather(const StepParams& p, int x, int y,
                                               int z, const float*, double (&f)[L::Q]) {
@@ -191,6 +197,16 @@ __device__ __noinline__ Check64 check_stored(const StepParams& p,
 // of neighbouring entries, of equal length, at most 32.
 __device__ __forceinline__ unsigned run_length(unsigned count, unsigned warps) {
   return min(32u, (count + warps - 1u) / warps);
+}
+// The run a warp takes.  Short lists: consecutive runs to different blocks, so
+// that every SM has some (dealt block by block, steps of 189 x 107 x 83 and of
+// the 12-member batch were 3 and 5 % longer).  Queues longer than the grid:
+// four consecutive runs to a block, which share cache lines and run on its
+// four sub-partitions (nodes that need the logarithms lie together, in a
+// symmetry plane).
+__device__ __forceinline__ unsigned dealt(bool bulk, unsigned warp) {
+  return bulk ? ((warp >> 2) * gridDim.x + blockIdx.x) * 4u + (warp & 3u)
+              : warp * gridDim.x + blockIdx.x;
 }
 
 // Open nodes per warp up to which they run one at a time (near64_warp) rather
@@ -243,7 +259,6 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
   const bool shifted = sizeof(S) == 2 || !p.unshifted;
   const int lane = threadIdx.x & 31;
   const unsigned W = gridDim.x * (blockDim.x >> 5);
-  const unsigned wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const LanePop lp = lane_pop<L>(lane);
   const bool bulk = count > gridDim.x * blockDim.x;
   Acc acc;
@@ -372,19 +387,19 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
     }
     return true;
   };
-  // this warp's pending nodes (warp-uniform counts): for the logarithms (on
-  // a queue longer than the grid) and for the series
-  // (8 warps; the series' list is below 32 before a round adds up to 32)
-  __shared__ unsigned pend_s[8][32], near_s[8][64];
+  // this warp's pending nodes (8 warps; warp-uniform counts): for the
+  // logarithms (on a queue longer than the grid; at most 32 before a round
+  // adds up to 32) and for the series (below 32 before)
+  __shared__ unsigned pend_s[8][64], near_s[8][64];
   const int warp = threadIdx.x >> 5;
   unsigned* pend = pend_s[warp];
   unsigned* near = near_s[warp];
   int npend = 0, nnear = 0;
-  auto flush = [&]() {   // every lane calls
+  auto flush = [&]() {   // 32 of them; every lane calls
+    npend -= 32;
     __syncwarp();
-    if (lane < npend) fp64_lane((long long)pend[lane]);
+    fp64_lane((long long)pend[npend + lane]);
     __syncwarp();
-    npend = 0;
   };
   // Nodes that need the logarithms (every lane calls).  Per lane a node
   // costs ~75 FP64 warp instructions of its warp (2,400 shared by 32 lanes),
@@ -392,11 +407,11 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
   // one per lane costs less FP64 issue in bulk.
   auto logarithms = [&](bool need64, long long node, bool near) {
     const unsigned m64 = __ballot_sync(0xffffffffu, need64);
-    if (CHECK ? !near : (!bulk && !near && __popc(m64) > 16)) {
+    if (CHECK ? !near : (!bulk && !near && __popc(m64) > 5)) {
       if (need64) fp64_lane(node);
     } else if (bulk && !near) {
       const int nk = __popc(m64);
-      if (npend + nk > 32) flush();
+      if (npend + nk > 64) flush();
       if (need64) pend[npend + __popc(m64 & ((1u << lane) - 1u))] =
           (unsigned)node;
       npend += nk;
@@ -436,14 +451,14 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
     bool need64 = false, open = false, direct = false, few = few_o;
     long long node = 0;
     if (base_o < open_count) {
-      const unsigned k = base_o +
-                         (blockIdx.x * use + (unsigned)warp) * run_o +
-                         (unsigned)lane;
+      const unsigned k =
+          base_o + dealt(bulk, (unsigned)warp) * run_o + (unsigned)lane;
       base_o += run_o * WO;
       direct = (unsigned)lane < run_o && k < open_count;
       if (direct) node = p.far_queue[p.far_cap - 1u - k];
     } else if (base_q < count) {
-      const unsigned k = base_q + wid * run_q + (unsigned)lane;
+      const unsigned k =
+          base_q + dealt(bulk, (unsigned)warp) * run_q + (unsigned)lane;
       base_q += run_q * W;
       if ((unsigned)lane < run_q && k < count) {
         const unsigned e = p.far_queue[k];
@@ -498,13 +513,32 @@ __global__ void __launch_bounds__(256) k_far_fixup(const StepParams p) {
     for (int t = 0; t < 2; ++t)
       logarithms(t == 0 ? direct : need64, t == 0 ? sn : node, t == 0 && few);
   }
-  if (npend > 0) {   // bulk remainder: few nodes run one per warp
-    __syncwarp();
-    if (npend > 5) {
-      flush();
-    } else {
-      Warp64 r;   // (with CHECK nothing is pending)
-      for (int j = 0; j < npend; ++j) fp64_warp((long long)pend[j], false, r);
+  // What the warps still hold of a long queue, pooled over the block: full
+  // warps of nodes, one per lane, on different sub-partitions (few nodes: one
+  // per warp).
+  if (bulk) {
+    __shared__ unsigned pool[8 * 64];
+    __shared__ int held[8];
+    if (lane == 0) held[warp] = npend;
+    __syncthreads();
+    int at = 0, total = 0;
+    for (int w = 0; w < 8; ++w) {
+      if (w < warp) at += held[w];
+      total += held[w];
+    }
+    for (int k = lane; k < npend; k += 32) pool[at + k] = pend[k];
+    __syncthreads();
+    for (int k = 32 * warp; k < total; k += 32 * 8) {
+      const int m = min(32, total - k);
+      const unsigned e = lane < m ? pool[k + lane] : 0u;
+      if (m > 5) {
+        if (lane < m) fp64_lane((long long)e);
+      } else {
+        for (int j = 0; j < m; ++j) {
+          Warp64 r;   // (with CHECK nothing is pending)
+          fp64_warp((long long)__shfl_sync(0xffffffffu, e, j), false, r);
+        }
+      }
     }
   }
   if (DIAG) acc.block_reduce_store(p.partials);

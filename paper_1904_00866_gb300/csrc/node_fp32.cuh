@@ -363,7 +363,8 @@ __device__ __forceinline__ void exact_moments(float d0,
 // equilibrium rounding, and the decision is retaken with the bounds of that
 // accuracy (series always to k = 8).  A node this leaves undecided is
 // flagged NF_FAR | NF_REFINE: its Delta H(2) lies within ~75 u of its own
-// scale, and the FP64 series (series64.cuh) settles it.  Writes
+// scale, and the FP64 series (series64.cuh) settles it; NF_FAR alone: it is
+// zero by symmetry, and the logarithms decide.  Writes
 // r.n0 / r.n2 (the more accurate n, used by the relaxation), r.alpha,
 // r.flags (NF_BAND set: the second stage decided) and the moments r.drho,
 // r.rho, r.j.
@@ -538,7 +539,12 @@ __device__ __forceinline__ void node32_refine(
   float alpha = 1.0f;
   const int k = decide32(h, alpha, kChordWidth);
   if (k == kUndecided) {
-    r.flags = NF_FAR | NF_REFINE;
+    // within the sum's own rounding of zero and below what the FP64 series
+    // settles (2^-45 M_2): a tie by symmetry (x ~ 1e-8 right after
+    // initialisation), whose series attempt is spared
+    r.flags = fabsf(h.D2) <= fminf(1.4e-14f, 8.0f * uu * xabs) * M[2]
+                  ? NF_FAR
+                  : NF_FAR | NF_REFINE;
     return;
   }
   r.alpha = alpha;
