@@ -87,10 +87,12 @@ ELBM_DECLARE_LAUNCHERS(d2q9)
 ELBM_DECLARE_LAUNCHERS(d3q27)
 #undef ELBM_DECLARE_LAUNCHERS
 
-// Second stage of the undecided D3Q27 nodes a step buffered (D2Q9 kernels
-// run it themselves).
+// Second stage of the undecided nodes a step buffered (D3Q27 and large
+// binary16 D2Q9 lattices; the other D2Q9 kernels run it themselves).
 cudaError_t launch_refine_d3q27(int diag, int check, const StepParams& p,
                                 int blocks, int grid, cudaStream_t s);
+cudaError_t launch_refine16_d2q9(int diag, int check, const StepParams& p,
+                                 int blocks, int grid, cudaStream_t s);
 cudaError_t launch_refine16_d3q27(int diag, int check, const StepParams& p,
                                   int blocks, int grid, cudaStream_t s);
 

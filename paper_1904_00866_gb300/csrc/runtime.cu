@@ -232,15 +232,24 @@ static elbm_status ensure_buffers(elbm_handle* h) {
     // sends the rest to the gathering queue, where each node costs ~3x more
     // (gather, FP32 stage again).  Half the nodes, at most 2^26 records
     // (8.6 GB) unless n / 16 is more, at least 65,536.  D2Q9 kernels run
-    // the second stage themselves.
-    if (h->q == 27) {
+    // the second stage themselves, but for large binary16 lattices, which
+    // gain: 1-2 % of their nodes are undecided, in nearly every warp, and each
+    // such warp would run all of it (FP32 shear layers: 76 %).  us per step,
+    // in the kernel / buffered, several flows: 512^2 15.8 / 17.0 and
+    // 16.5 / 20.0, 1024^2 43.6 / 37.2, 46.2 / 39.9, 48.9 / 41.1, 40.0 / 39.5
+    // and 35.7 / 38.7, 2000^2 140.5 / 112.1 and 128.6 / 113.8.
+    const bool buffered =
+        h->q == 27 || (h->dtype == ELBM_FP16_SHIFTED && h->n > (1 << 19));
+    if (buffered) {
       const long long cap = std::min<long long>(
           h->n, std::max<long long>(
                     65536, std::min<long long>(
                                h->n / 2, std::max<long long>(h->n / 16,
                                                              1LL << 26))));
       h->refine_buf = (float*)dev_alloc(
-          h, sizeof(float) * (size_t)refine_record<D3Q27>() * (size_t)cap);
+          h, sizeof(float) * (size_t)(h->q == 27 ? refine_record<D3Q27>()
+                                                 : refine_record<D2Q9>()) *
+                 (size_t)cap);
       h->refine_counts =
           (unsigned*)dev_alloc(h, sizeof(unsigned) * kMaxRefineBlocks);
       h->refine_cap = h->refine_buf && h->refine_counts ? (unsigned)cap : 0u;
@@ -680,8 +689,8 @@ elbm_status elbm_step(elbm_handle* h, long long nsteps, elbm_alpha_mode mode) {
       if (p.exact && p.refine_cap) {
         // second stage of the undecided nodes the step buffered
         pf.partials = h->partials + (size_t)rows * NSTAT;
-        e = storage == 2 ? launch_refine16_d3q27(diag, check, pf, grid, fgrid,
-                                                 h->stream)
+        e = storage == 2 ? (d2 ? launch_refine16_d2q9 : launch_refine16_d3q27)(
+                               diag, check, pf, grid, fgrid, h->stream)
                          : launch_refine_d3q27(diag, check, pf, grid, fgrid,
                                                h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "second stage launch");

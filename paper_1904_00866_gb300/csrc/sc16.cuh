@@ -93,15 +93,17 @@ __global__ void __launch_bounds__(kSc32Threads, 2)
           in, rho0f, p.rho0, beta, 0.0f, nullptr,
           p.alpha_map ? p.alpha_map + node : nullptr, acc,
           out, p.exact ? &ap : nullptr);
-    // D2Q9: the second stage here, as in k_sc32
+    // D2Q9 without a record buffer (small lattices): the second stage here, as
+    // in k_sc32
+    bool here = false;
     if constexpr (Q == 9) {
-      if (p.exact)
+      here = p.refine_cap == 0u;
+      if (p.exact && here)
         st = refine_inline<L, true, DIAG, CHECK>(p, in, node, st, ap, acc,
                                                  out);
-    } else {
-      if (p.exact)
-        defer_undecided<L>(p, &s_refine, st == kNodeRefine, in, node, ap);
     }
+    if (p.exact && !here)
+      defer_undecided<L>(p, &s_refine, st == kNodeRefine, in, node, ap);
     defer_nodes(&p.far_count[p.parity], p.far_queue, p.far_cap, p.err_flags,
                 node, st == kNodeFar ? kNodeFar : kNodeDone);
   }
