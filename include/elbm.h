@@ -69,7 +69,12 @@ typedef struct elbm_handle elbm_handle;
 typedef enum { ELBM_D2Q9 = 0, ELBM_D3Q27 = 1, ELBM_D1Q3 = 2 } elbm_lattice;
 
 /* Storage (and arithmetic) of the populations.
- *   ELBM_FP64          f_i in FP64, FP64 arithmetic throughout.
+ *   ELBM_FP64          f_i, moments, equilibrium and relaxation in FP64.  The
+ *                      entropy differences of Eqs. (4) and (9) by FP64
+ *                      logarithms, or near equilibrium (max |x_i| <= 1/48)
+ *                      by a moment series whose terms are pairs of FP32
+ *                      numbers (FP32 from the seventh on): alpha to about
+ *                      1e-15, as the logarithms give it.
  *   ELBM_FP32          f_i in FP32.
  *   ELBM_FP32_SHIFTED  delta_i = f_i - W_i rho0 in FP32 (rho0 a per-handle
  *                      constant, the FP32-rounded mean initial density).
@@ -81,8 +86,9 @@ typedef enum { ELBM_D2Q9 = 0, ELBM_D3Q27 = 1, ELBM_D1Q3 = 2 } elbm_lattice;
  *                      and momentum are conserved to that rounding only.
  * FP32 and FP16 storages compute FORMULA in FP32 with a certified error bound
  * on the entropy differences (see elbm_step) applied to the values as
- * loaded; ROOT and SECANT, and nodes far from equilibrium, are computed in
- * FP64 from the stored values. */
+ * loaded; ROOT and SECANT, and nodes far from equilibrium, are computed as
+ * for FP64 storage from the stored values (the series up to 1/32), with alpha
+ * rounded down to FP32. */
 typedef enum {
   ELBM_FP64 = 0,
   ELBM_FP32 = 1,
@@ -101,9 +107,9 @@ typedef enum {
  * bound).
  *   ELBM_DECISION_EXACT (default): a second stage recomputes f^eq - f in
  *     double-float arithmetic and retakes the acceptance test after Eq. (8)
- *     and Eq. (9) with that error bound (then with the leading terms of
- *     Delta H(2) in double-float as well, and FP64 for the rare node still
- *     undecided), so every node takes the branch the exact arithmetic
+ *     and Eq. (9) with that error bound (then by the moment series of FP64
+ *     storage, and by FP64 logarithms where Delta H(2) lies within rounding
+ *     of zero), so every node takes the branch the exact arithmetic
  *     takes and an Eq. (9) alpha lies within 2^-16 of the chord of the
  *     stored state: alpha and the Fig. 5 counter are the paper's.  Costs
  *     about 10 % per step on developed 3D flows, more where most nodes are
@@ -134,7 +140,12 @@ typedef enum {
 } elbm_status;
 
 /* Diagnostics of one step (the step that maps f^n to f^{n+1}): moments and
- * entropy of f^n and counters of the collisions performed. */
+ * entropy of f^n and counters of the collisions performed.  FP64 storage, ROOT
+ * and SECANT: each node's moments in FP64, summed in FP64.  FP32 / FP16
+ * FORMULA: each node's rho - rho0 and rho u as FP32 numbers and its kinetic
+ * energy from them, in compensated FP32 sums per thread and FP64 sums over
+ * threads; nodes of the second stage are summed (and their kinetic energy
+ * formed) as exactly as in FP64, nodes solved in FP64 enter in FP64. */
 typedef struct {
   long long step;           /* n                                          */
   long long n_nodes;
@@ -151,7 +162,8 @@ typedef struct {
   long long n_far;          /* FP32 FORMULA: node solved in FP64 (far from
                                equilibrium, invalid, or Delta H(2) within
                                its rounding of zero)                      */
-  long long n_degenerate;   /* f^eq == f: alpha = 2                       */
+  long long n_degenerate;   /* f^eq == f in the evaluation's precision:
+                               alpha = 2                                  */
   long long n_root_iters;   /* ROOT/SECANT iterations                     */
   long long n_root_cap;     /* ROOT stopped at the iteration cap          */
   long long n_no_root;      /* ROOT: Delta H(alpha_max) <= 0, alpha_max   */
@@ -159,7 +171,9 @@ typedef struct {
   int reserved;
   double h_total;           /* sum_x H(f^n(x)), Eq. (3), FP64             */
   long long n_violations;   /* nodes with Delta H(alpha) above its FP64
-                               rounding bound (Eq. (7) violated)          */
+                               rounding bound (Eq. (7) violated), at the
+                               alpha the step took; the check itself uses
+                               FP64 logarithms                            */
   long long n_decision_mismatch; /* FP32 accept/formula decision differs
                                from the FP64 one (nodes where f = f^eq at
                                the evaluation's precision -- the update
@@ -236,8 +250,8 @@ ELBM_API elbm_status elbm_set_populations(elbm_handle *h, const double *f);
  * upper bounds and rounded down, is taken when Delta H(2) - E > 0 and
  * Delta H(1) + E < 0.  A node where either sign lies within E is
  * recomputed in double-float arithmetic (f^eq - f to about 1e-12 of f) and
- * decided again with that smaller error; the rare node still undecided is
- * solved in FP64.  So each node takes the branch of the exact arithmetic
+ * decided again with that smaller error; a node still undecided takes the
+ * FP64 moment series or logarithms.  So each node takes the branch of the exact arithmetic
  * and H(f*(alpha)) <= H(f) holds for the stored state.  Nodes with
  * max|x_i| > 1/8, |u_a| >= 1/4 or invalid populations are solved in FP64.
  * FP32 and FP16 storages take fewer than 2^31 nodes. */

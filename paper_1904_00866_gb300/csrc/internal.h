@@ -17,8 +17,9 @@ void count_launches(long long n);
 // and its blocks may be scheduled while that kernel's last ones run
 // (programmatic dependent launch); they wait there until it has completed
 // and its writes are visible, so only the launch latency overlaps.  us per
-// step (GB300), before -> with it: D3Q27 32^3 FP32 (four kernels) 36 -> 26,
-// D2Q9 64^2 FP64 (two) 12.3 -> 9.7, D3Q27 96^3 111 -> 104.
+// step (GB300), without -> with it, three flows: D2Q9 64^2 FP64 (two kernels)
+// 12.3 -> 9.7; D3Q27 32^3 FP32 (four) 38-40 -> 35.5; D3Q27 96^3 108 -> 103;
+// D2Q9 1024^2 shear layer 67-68 -> 64.
 template <class... P, class... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), int grid, int block,
                                   size_t smem, cudaStream_t s, int chained,
@@ -43,8 +44,8 @@ inline cudaError_t launch_chained(void (*kernel)(P...), int grid, int block,
 void set_global_error(const std::string& msg);
 
 // Whether the kernels of a step over `bytes` of populations are chained: up
-// to 128 MB.  Small steps gain the launch latency (D3Q27 32^3, 3.5 MB: 27 %;
-// 96^3, 96 MB: 4 %); beyond, it is below 3 % of the step, and the next
+// to 128 MB.  Small steps gain the launch latency (D2Q9 64^2: 21 %; D3Q27 32^3,
+// 3.5 MB: 6-11 %; 96^3, 96 MB: 5 %); beyond, it is below 3 % of the step, and the next
 // kernel's waiting blocks cost more than that (D3Q27 189 x 107 x 83, 181 MB:
 // 2.88 ms per 20 steps without, 2.97 with; the batch's steps 4.64 and 5.25,
 // so its launches are never chained).

@@ -166,10 +166,10 @@ __host__ __device__ constexpr bool pair_order() {
 // one chain per sum) and 6 for D2Q9 (10).
 //
 // Three such sums, the projection's single rounding and the maxima per
-// weight class take 59 of ~450 packed operations off a D3Q27 node, whose
-// kernels are bound by them.  us per pass, before -> after (GB300): 512^3
-// FP32, 8 steps 51380 -> 50610; 256^3 binary16, 8 steps 7175 -> 6809;
-// 189 x 107 x 83 with statistics, 20 steps 2877 -> 2770.
+// weight class take 59 of ~450 packed operations off a D3Q27 node.  us per
+// pass on one flow, both builds in turn (GB300): 512^3 FP32, 8 steps
+// 51360 -> 50610; 256^3 binary16, 8 steps 7173 -> 6798; 189 x 107 x 83 with
+// statistics, 20 steps 2879 -> 2760; 12-member batch, 32 steps 4636 -> 4525.
 template <class L>
 __device__ __forceinline__ void moments2(float v0,
                                          const float2 (&vv)[npairs<L>()],
